@@ -188,7 +188,8 @@ class Clocks:
                 "samples": len(rows), "reasons": reasons}
 
 
-STAGE_SOURCES = ["stage_kernel.cuh", "stage.cu", "stage_tiles.cu", "su3.cuh", "expm.cuh", "lattice.cuh"]
+STAGE_SOURCES = ["stage_kernel.cuh", "stage.cu", "stage_tiles.cu", "stage64.cuh", "stage64.cu", "fixed.cuh", "planes.cuh",
+                 "su3.cuh", "expm.cuh", "lattice.cuh"]
 
 
 def stage_source_hash():

@@ -485,7 +485,7 @@ tgf_status tgf_check_errors(unsigned* bits) {
     if (!bits) return fail(TGF_EINVAL, "bits is NULL");
 #ifdef TGF_CHECK
     TGF_CUDA(cudaDeviceSynchronize());
-    const unsigned w[6] = {check_word_stage(), check_word_measure(), check_word_pack(), check_word_mc(),
+    const unsigned w[6] = {check_word_stage() | check_word_stage64(), check_word_measure(), check_word_pack(), check_word_mc(),
                            check_word_sun(), check_word_stage_tiles()};
     unsigned b = 0;
     for (int i = 0; i < 6; ++i)

@@ -1,0 +1,362 @@
+// fixed.cuh -- products of unitary matrices in 58-bit fixed point on the integer pipe.
+//
+// Why.  GB300 issues a warp's FP64 FMA every 64 cycles per SM quarter, but a 32 x 32 + 64 -> 64 bit
+// integer multiply-add (IMAD.WIDE) every 4 (measured: 1.90 and 29 lanes per clock and SM).
+// Entries of SU(N) matrices are at most 1, so they need no exponent: an entry is the integer
+// v = floor(x 2^58), split as v = hi 2^29 + lo with 0 <= lo < 2^29, and one multiply-add of two
+// entries is three IMAD.WIDE (hi hi; hi lo and lo hi, summed apart; lo lo is below the last bit kept):
+// 13 cycles instead of 64.
+//
+// Accuracy.  Sums are exact: rounding enters once per entry and product, when the sum of the cross
+// terms is rounded to a multiple of 2^-55 (error at most 2^-56 = 1.4e-17), and once when an
+// operand is taken in (below 2^-57).  In FP64 the same entry, a sum of 2N products of size up to 1,
+// carries up to 2N roundings of 2^-54.  So a staple formed here is nearer to its exact value
+// than one formed in FP64.
+//
+// Range.  Nothing wraps as long as operand entries stay within the bounds noted at each split: with
+// 2N <= 8 terms of a link and another operand, hi hi sums stay below 8 x 2^30 x 2^29.01 and cross sums
+// below 8 (2^30 2^29 + 2^29.01 2^29), both under 2^63.  The
+// fields are arbitrary user data, so every operand is checked as it is taken in: a link entry
+// above 1 + 2^-10 in magnitude (also infinities and NaN), a product T above 2, a staple sum above 8
+// set bits in a guard word; a thread that finds them set repeats its link in FP64 arithmetic, which
+// takes any input.  SU(N) fields never do.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "lattice.cuh"
+#include "su3.cuh"
+
+namespace tgf {
+
+// (hi 2^29 + lo) in units that depend on the operand: 2^-58 for links and T (SPLIT 0), 2^(SH-58)
+// for wider operands split with SH > 0
+template <int N>
+struct matx {
+    int rh[N][N], rl[N][N], ih[N][N], il[N][N];
+};
+// sums of products
+template <int N>
+struct matq {
+    long long re[N][N], im[N][N];
+};
+
+constexpr int kFxBits = 58;
+
+
+struct fx_guard {
+    unsigned top = 0;   // bit 31: an operand outside its bound
+    unsigned top2 = 0;  // bits 30, 31: a staple sum outside its bound
+    __device__ __forceinline__ bool bad() const { return ((top >> 31) | (top2 >> 30)) != 0; }
+};
+
+// x -> floor(x 2^58) (negative x: to within one unit, as the bitwise complement of |x|'s image) split
+// into hi, lo.  The mantissa with its leading bit is aligned at the top of 64 bits and
+// shifted right by 1025 - exponent, which leaves x 2^61; shifts past 63 bits give 0.
+// `up` takes x 2^up instead (a matrix of small entries keeps its relative precision).
+__device__ __forceinline__ void fx_take(double x, int& hi, int& lo, fx_guard& g, unsigned up = 0) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const unsigned a = h & 0x7fffffffu;
+    g.top |= (0x3FF00400u - (up << 20)) - a;  // |x| 2^up <= 1 + 2^-10, else bit 31
+    const unsigned s = (1025u - up) - (a >> 20);
+    unsigned long long m = ((unsigned long long)(__funnelshift_l(l, h, 11) | 0x80000000u) << 32) | (l << 11);
+    asm("shr.b64 %0, %0, %1;" : "+l"(m) : "r"(s));
+    const int sg = (int)h >> 31;
+    asm("xor.b32 %0, %1, %2;" : "=r"(hi) : "r"((int)(m >> 32)), "r"(sg));
+    asm("shr.u32 %0, %1, 3;" : "=r"(lo) : "r"((unsigned)m ^ (unsigned)sg));
+}
+
+// a sum (units 2^-58) -> operand in units 2^(SH-58); |v| < 2 (SH = 0), 4 (SH = 1) or 8 (SH = 2)
+template <int SH>
+__device__ __forceinline__ void fx_split(long long v, int& hi, int& lo) {
+    asm("{.reg .b64 t; shr.s64 t, %1, %2; cvt.u32.u64 %0, t;}" : "=r"(hi) : "l"(v), "n"(29 + SH));
+    asm("and.b32 %0, %1, 0x1fffffff;" : "=r"(lo) : "r"((int)(v >> SH)));
+}
+
+template <int N>
+__device__ __forceinline__ void fx_zero(matq<N>& a) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) a.re[i][j] = a.im[i][j] = 0;
+}
+
+// a wider operand; its bound (2^(SH+1)) must have been checked
+template <int N, int SH>
+__device__ __forceinline__ void fx_operand_wide(matx<N>& o, const matq<N>& v) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            fx_split<SH>(v.re[i][j], o.rh[i][j], o.rl[i][j]);
+            fx_split<SH>(v.im[i][j], o.ih[i][j], o.il[i][j]);
+        }
+}
+// |entries| < 8 (B = 29) or 4 (B = 28), else the guard's second word
+template <int N, int B>
+__device__ __forceinline__ void fx_check(const matq<N>& v, fx_guard& g) {
+    constexpr int up = 29 - B;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            g.top2 |= (((unsigned)(int)(v.re[i][j] >> 32) + (1u << B)) | ((unsigned)(int)(v.im[i][j] >> 32) + (1u << B))) << up;
+}
+
+// c + a b by one IMAD.WIDE.  Written as C++: mad.wide in PTX becomes a product and a separate 64-bit
+// addition.  The compiler must not see that lo is never negative nor where hi comes from (their last instruction is
+// therefore inline assembly): a zero-extended factor times a sign-extended one would become a full
+// 64 x 64 bit product.
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return c + (long long)a * b; }
+__device__ __forceinline__ int fx_neg(int a) { return (int)(0u - (unsigned)a); }
+__device__ __forceinline__ void fx_mad(long long& hh, long long& cr, int ah, int al, int bh, int bl) {
+    hh = mad_wide(ah, bh, hh);
+    cr = mad_wide(ah, bl, cr);
+    cr = mad_wide(al, bh, cr);
+}
+// start of a cross sum: its top word is then the rounded one (opaque: an accumulator of the first
+// multiply-add, not an addition of its own)
+__device__ __forceinline__ long long fx_round() {
+    long long r;
+    asm("mov.b64 %0, 0x80000000;" : "=l"(r));
+    return r;
+}
+// hi hi sum + rounded cross sum: the cross unit is 2^-29 of the hi hi unit, its top word 8 of them
+__device__ __forceinline__ long long fx_join(long long hh, long long cr) { return mad_wide((int)(cr >> 32), 8, hh); }
+
+// Re and Im of c + sum_k a_k w_k, w = b or (CONJ) its complex conjugate; minus signs go to a negated copy of a
+// (lo < 2^29, so -lo is exact).
+template <int N>
+struct vecx {
+    int rh[N], rl[N], ih[N], il[N];
+};
+template <int N, bool CONJ>
+__device__ __forceinline__ void fx_dot(long long& re, long long& im, const vecx<N>& a, const vecx<N>& na, const vecx<N>& b,
+                                       long long half) {
+    long long rc = half, ic = half;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        fx_mad(re, rc, a.rh[k], a.rl[k], b.rh[k], b.rl[k]);
+        if (CONJ) {
+            fx_mad(im, ic, a.ih[k], a.il[k], b.rh[k], b.rl[k]);
+            fx_mad(re, rc, a.ih[k], a.il[k], b.ih[k], b.il[k]);
+            fx_mad(im, ic, na.rh[k], na.rl[k], b.ih[k], b.il[k]);
+        } else {
+            fx_mad(im, ic, a.rh[k], a.rl[k], b.ih[k], b.il[k]);
+            fx_mad(re, rc, na.ih[k], na.il[k], b.ih[k], b.il[k]);
+            fx_mad(im, ic, a.ih[k], a.il[k], b.rh[k], b.rl[k]);
+        }
+    }
+    re = fx_join(re, rc);
+    im = fx_join(im, ic);
+}
+template <int N>
+__device__ __forceinline__ vecx<N> fx_negated(const vecx<N>& a) {
+    vecx<N> n;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        n.rh[k] = fx_neg(a.rh[k]);
+        n.rl[k] = fx_neg(a.rl[k]);
+        n.ih[k] = fx_neg(a.ih[k]);
+        n.il[k] = fx_neg(a.il[k]);
+    }
+    return n;
+}
+template <int N>
+__device__ __forceinline__ vecx<N> fx_row(const matx<N>& m, int i) {
+    vecx<N> v;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        v.rh[k] = m.rh[i][k];
+        v.rl[k] = m.rl[i][k];
+        v.ih[k] = m.ih[i][k];
+        v.il[k] = m.il[i][k];
+    }
+    return v;
+}
+template <int N>
+__device__ __forceinline__ vecx<N> fx_col(const matx<N>& m, int j) {
+    vecx<N> v;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        v.rh[k] = m.rh[k][j];
+        v.rl[k] = m.rl[k][j];
+        v.ih[k] = m.ih[k][j];
+        v.il[k] = m.il[k][j];
+    }
+    return v;
+}
+
+// c = a b
+template <int N>
+__device__ __forceinline__ void fx_mul_nn(matq<N>& c, const matx<N>& a, const matx<N>& b) {
+    const long long half = fx_round();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const vecx<N> r = fx_row(a, i), nr = fx_negated(r);
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            c.re[i][j] = c.im[i][j] = 0;
+            fx_dot<N, false>(c.re[i][j], c.im[i][j], r, nr, fx_col(b, j), half);
+        }
+    }
+}
+
+// c *= exp(2 pi i k / 3) or its conjugate (zr + i zi): once in a while, at the twisted corner
+template <int N>
+__device__ __forceinline__ void fx_scale(matx<N>& m, double zr, double zi) {
+    fx_guard g;
+    const long long half = fx_round();
+    int zrh, zrl, zih, zil;
+    fx_take(zr, zrh, zrl, g);
+    fx_take(zi, zih, zil, g);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            long long rh = 0, ih = 0, rc = half, ic = half;
+            fx_mad(rh, rc, m.rh[i][j], m.rl[i][j], zrh, zrl);
+            fx_mad(rh, rc, fx_neg(m.ih[i][j]), fx_neg(m.il[i][j]), zih, zil);
+            fx_mad(ih, ic, m.rh[i][j], m.rl[i][j], zih, zil);
+            fx_mad(ih, ic, m.ih[i][j], m.il[i][j], zrh, zrl);
+            fx_split<0>(fx_join(rh, rc), m.rh[i][j], m.rl[i][j]);
+            fx_split<0>(fx_join(ih, ic), m.ih[i][j], m.il[i][j]);
+        }
+}
+
+template <int N>
+__device__ __forceinline__ void fx_take_entry(matx<N>& o, int i, int j, double re, double im, fx_guard& g, unsigned up = 0) {
+    fx_take(re, o.rh[i][j], o.rl[i][j], g, up);
+    fx_take(im, o.ih[i][j], o.il[i][j], g, up);
+}
+
+// ---- staple sums ------------------------------------------------------------------------------
+//
+// Both staples of a direction are one computation.  With V, B, C the three links,
+//   forward   F = Z*_{mu nu}(n) U_nu(n+mu) U_mu(n+nu)^+ U_nu(n)^+:
+//             row i of F = conj-dot of (row i of V, rows of B) with the rows of C,  V = U_nu(n+mu), B = U_mu(n+nu), C = U_nu(n)
+//   backward  G = Z_{mu nu}(n-nu) U_nu(n+mu-nu)^+ U_mu(n-nu)^+ U_nu(n-nu):
+//             column j of G is the same expression of the transposed links V = U_nu(n-nu), B = U_mu(n-nu), C = U_nu(n+mu-nu)
+// so one loop body serves both, reading the backward links transposed (an address choice) and summing onto the
+// transposed staple sum, which is transposed in registers between the two.  The body of about 1500
+// instructions stays in the instruction cache, where two would not, and only B, C, the sum and one row
+// are live, so that 12 warps fit on an SM instead of 8.
+//
+// SRC: get(dir, site, i, j, tr) loads entry (i, j), transposed if tr (a value uniform over the warp).
+// SYNC: a block barrier per iteration (every thread of the block must be here).  The warps of a block then
+// fetch the same instructions at the same time: 11 % on the FP64 stage (8.63 instead of 9.74 ms for
+// 4 steps of 4 x 8x8x24x24).
+// visit(q, nu, sig): called after the forward (q = 0) and after the backward staple (q = 1) of a direction,
+// with the sum in normal orientation; skip(nu) leaves a direction out.
+template <int N>
+__device__ __forceinline__ void fx_transpose(matq<N>& m) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = i + 1; j < N; ++j) {
+            const long long r = m.re[i][j], q = m.im[i][j];
+            m.re[i][j] = m.re[j][i];
+            m.im[i][j] = m.im[j][i];
+            m.re[j][i] = r;
+            m.im[j][i] = q;
+        }
+}
+
+template <int N, class SRC>
+__device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, int site, bool tr, fx_guard& g) {
+    double2 x[N][N];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) x[i][j] = src.get(dir, site, i, j, tr);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) fx_take_entry<N>(o, i, j, x[i][j].x, x[i][j].y, g);
+}
+
+template <int N, bool SYNC, class SRC, class SKIP, class VISIT>
+__device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const CfgDesc& c, int s, int mu, unsigned eb, fx_guard& g,
+                                           SKIP&& skip, VISIT&& visit) {
+    const int s_mp = fwd(c, eb, s, mu);
+    const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
+    const long long half = fx_round();
+#pragma unroll 1
+    for (int q = 0; q < 6; ++q) {
+        const bool back = q & 1;
+        const int nu = (mu + 1 + (q >> 1)) & 3;
+        if (SYNC) __syncthreads();
+        if (skip(nu)) continue;
+        const int s_nm = bwd(c, eb, s, nu);
+        const int sb = back ? s_nm : fwd(c, eb, s, nu);
+        const int sv = back ? s_nm : s_mp;
+        const int sc = back ? fwd(c, eb, s_nm, mu) : s;  // x_mu(n - nu) = x_mu(n)
+        if (back) fx_transpose(sig);
+        matx<N> b, d;
+        fx_take_matrix<N>(b, src, mu, sb, back, g);
+        // the twisted corner's centre factor goes to B: Z* V B^+ = V (Z B)^+
+        const int k = c.tw[mu * 4 + nu];
+        if (k != 0 && at_mu0 && ((eb >> (back ? 8 + nu : nu)) & 1u)) {
+            double zr, zi;
+            SRC::centre(k, zr, zi);
+            fx_scale(b, zr, back ? -zi : zi);
+        }
+        fx_take_matrix<N>(d, src, nu, sc, back, g);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            vecx<N> v, t;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const double2 x = src.get(nu, sv, i, j, back);
+                fx_take(x.x, v.rh[j], v.rl[j], g);
+                fx_take(x.y, v.ih[j], v.il[j], g);
+            }
+            vecx<N> nv = fx_negated(v);
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                long long re = 0, im = 0;
+                fx_dot<N, true>(re, im, v, nv, fx_row(b, j), half);
+                fx_split<0>(re, t.rh[j], t.rl[j]);
+                fx_split<0>(im, t.ih[j], t.il[j]);
+                g.top |= (unsigned)(t.rh[j] + (1 << 30)) | (unsigned)(t.ih[j] + (1 << 30));
+            }
+            nv = fx_negated(t);
+#pragma unroll
+            for (int j = 0; j < N; ++j) fx_dot<N, true>(sig.re[i][j], sig.im[i][j], t, nv, fx_row(d, j), half);
+        }
+        if (back) fx_transpose(sig);
+        fx_check<N, 29>(sig, g);
+        visit(q & 1, nu, sig);
+    }
+}
+
+// FP64 links for fixed.cuh: entry e of a link at base + (e / 2) 4 Vp + 4 s + 2 (e % 2), entry 8 at 16 Vp + 2 s
+struct Su3Src {
+    const double* base;
+    int Vp;
+    __device__ __forceinline__ double2 get(int dir, int s, int i, int j, bool tr) const {
+        s = checked_site(s, Vp);
+        const double* p = base + (size_t)dir * 18 * Vp;
+        if (i == 2 && j == 2) return __ldg(reinterpret_cast<const double2*>(p + (size_t)16 * Vp) + s);
+        const int e = 3 * i + j, f = 3 * j + i;
+        const int oe = (e >> 1) * 4 * Vp + (e & 1) * 2, of = (f >> 1) * 4 * Vp + (f & 1) * 2;
+        return __ldg(reinterpret_cast<const double2*>(p + (size_t)(tr ? of : oe) + (size_t)s * 4));
+    }
+    static __device__ __forceinline__ void centre(int k, double& zr, double& zi) { tgf::centre<double>(k, zr, zi); }
+};
+
+// The largest up <= 40 for which every entry of m stays below 1 in magnitude times 2^up.
+__device__ __forceinline__ unsigned fx_scale_of(const mat3<double>& m) {
+    unsigned a = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            a = max(a, (unsigned)__double2hiint(m.e[i][j].re) & 0x7fffffffu);
+            a = max(a, (unsigned)__double2hiint(m.e[i][j].im) & 0x7fffffffu);
+        }
+    return (unsigned)min(max(1022 - (int)(a >> 20), 0), 40);
+}
+
+}  // namespace tgf

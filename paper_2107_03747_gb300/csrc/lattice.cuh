@@ -157,6 +157,7 @@ __device__ __forceinline__ int checked_site(int s, int) { return s; }
 // per translation unit check words of a self-checking build
 unsigned check_word_stage();
 unsigned check_word_stage_tiles();
+unsigned check_word_stage64();
 unsigned check_word_measure();
 unsigned check_word_pack();
 unsigned check_word_mc();
@@ -404,6 +405,8 @@ void launch_stage(int prec, int stage, int mode, int reunit, const Batch& B, con
                   void* acc, void* clov, cudaStream_t st, int grid = 0, int tile = 0);
 void launch_stage_tile(int tile, int prec, int stage, int mode, int reunit, const Batch& B, const void* w_in,
                        void* w_out, void* acc, void* clov, cudaStream_t st, int grid);
+void launch_stage64(int stage, int mode, const Batch& B, const double* w_in, double* w_out, double* acc, double* clov,
+                    cudaStream_t st, int grid);
 constexpr int kTiles = 5;
 inline int tile_sites(int tile) { return tile == 1 ? 64 : 32; }
 void launch_clover_sum(int prec, unsigned flags, const Batch& B, const void* clov, double* partial,

@@ -1,0 +1,244 @@
+// stage64.cuh -- one RK3 stage, the clover halves, or both, in double precision: links, the accumulator
+// X and the exponential in FP64, the matrix products in 58-bit fixed point on the integer pipe
+// (fixed.cuh).
+//
+// With every product in FP64 the stage kept the FP64 pipe 94-97 % busy (107,000 cycles per warp and SM
+// quarter), and nothing else of the chip was in use.  Here that pipe carries the exponential and the
+// conversions (about 290 instructions, 19,000 cycles), the integer pipe 13 products (4,700 IMAD.WIDE
+// of 4 cycles) and the splitting of the operands, side by side: 36,000 cycles.  4 steps of
+// 4 x 8x8x24x24, measured each step: 23.7 ms before, 8.6 now; one measurement of 4 x 7x7x21x21: 693 us
+// before, 312 now; 3 steps of 4x4x12x12 (latency): 696 us before, 392 now.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "expm.cuh"
+#include "fixed.cuh"
+#include "lattice.cuh"
+#include "planes.cuh"
+
+namespace tgf {
+
+// the anti-Hermitian part D - D^+ of a product (units `unit`), as store_ah
+__device__ __forceinline__ void fx_store_ah(double* __restrict__ p, int Vp, int s, const matq<3>& d, double unit) {
+    const double v[9] = {2 * unit * (double)d.im[0][0],          2 * unit * (double)d.im[1][1],
+                         2 * unit * (double)d.im[2][2],          unit * (double)(d.re[0][1] - d.re[1][0]),
+                         unit * (double)(d.im[0][1] + d.im[1][0]), unit * (double)(d.re[0][2] - d.re[2][0]),
+                         unit * (double)(d.im[0][2] + d.im[2][0]), unit * (double)(d.re[1][2] - d.re[2][1]),
+                         unit * (double)(d.im[1][2] + d.im[2][1])};
+    AhStore<double>::store(p, Vp, s, v);
+}
+
+// X of stage STAGE from the force z, with the accumulator read and written where the stage does.
+template <int STAGE>
+__device__ __forceinline__ void rk3_x(alg8<double>& x, const alg8<double>& z, double h, double* xb, int Vp, int s) {
+    if (STAGE == 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x.v[i] = 0.25 * h * z.v[i];
+    } else {
+        AccStore<double>::load(xb, Vp, s, x);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            x.v[i] = STAGE == 2 ? (8.0 / 9.0) * h * z.v[i] - (17.0 / 9.0) * x.v[i] : 0.75 * h * z.v[i] - x.v[i];
+    }
+    if (STAGE != 3) AccStore<double>::store(xb, Vp, s, x);
+}
+
+// The force (and the clover halves) in FP64 throughout, for links whose fields leave the range of
+// fixed.cuh (entries above 1 + 2^-10, infinities, NaN): any input, at the FP64 pipe's rate.
+template <int MODE>
+__device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c, const double* __restrict__ base,
+                                               double* __restrict__ cb, int s, int mu, unsigned eb) {
+    const int Vp = c.Vp;
+    auto link = [&](int dir, int site, mat3<double>& u) { Store<P64>::load(base + (size_t)dir * 18 * Vp, Vp, site, u); };
+    mat3<double> sig, a, b, t, f;
+    set_zero(sig);
+    const int s_mp = fwd(c, eb, s, mu);
+    const bool at_mu0 = (eb >> mu) & 1u;
+#pragma unroll 1
+    for (int dn = 1; dn < 4; ++dn) {
+        const int nu = (mu + dn) & 3;
+        const bool clover = MODE != 0 && c_clover_owner[mu][nu];
+        if (MODE == 2 && !clover) continue;
+        const int s_nm = bwd(c, eb, s, nu);
+        const int k = c.tw[mu * 4 + nu];
+        double zr = 1.0, zi = 0.0;
+        if (k != 0) centre<double>(k, zr, zi);
+        link(nu, s_mp, a);
+        link(mu, fwd(c, eb, s, nu), b);
+        mul_nd(t, a, b);
+        link(nu, s, a);
+        mul_nd(f, t, a);
+        if (k != 0 && at_mu0 && ((eb >> nu) & 1u)) scale_cx(f, zr, -zi);
+        add_to(sig, f);
+        link(mu, s_nm, a);
+        link(nu, fwd(c, eb, s_nm, mu), b);
+        mul_nn(t, a, b);
+        link(nu, s_nm, a);
+        mul_dn(b, t, a);
+        if (k != 0 && at_mu0 && ((eb >> (8 + nu)) & 1u)) scale_cx(b, zr, zi);
+        add_to(sig, b);
+        if (clover) {
+            const int pl = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
+            link(mu, s, a);
+            double rt = 0.0;
+            const double sg = nu > mu ? 1.0 : -1.0;
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    rt = fma(a.e[i][j].re, f.e[j][i].re, fma(-a.e[i][j].im, f.e[j][i].im, rt));
+            cb[(size_t)(108 + pl) * Vp + s] = 3.0 - rt;
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    f.e[i][j].re = sg * (f.e[i][j].re - b.e[i][j].re);
+                    f.e[i][j].im = sg * (f.e[i][j].im - b.e[i][j].im);
+                }
+            mul_nn(t, a, f);
+            store_ah(cb + (size_t)(pl * 2 + 0) * 9 * Vp, Vp, s, t);
+            mul_nn(t, f, a);
+            store_ah(cb + (size_t)(pl * 2 + 1) * 9 * Vp, Vp, s_mp, t);
+        }
+    }
+    if (MODE == 2) return;
+    link(mu, s, a);
+    mul_nn(t, a, sig);
+    minus_proj_ta(z, t);
+}
+
+// One thread per link; a block covers 32 sites x 4 directions, warps grouped by mu.  MODE as in k_stage:
+// 0 the stage, 1 the stage and the clover halves of the input field, 2 the halves only.
+template <int STAGE, int MODE, int CAP>
+__global__ void __launch_bounds__(128, MODE == 0 ? 3 : 2)
+k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
+          double* __restrict__ acc, double* __restrict__ clov) {
+    const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
+        const int ci = find_cfg(B, blk);
+        const CfgDesc& c = B.c[ci];
+        int s = (blk - c.blk0) * 32 + lane;
+        const bool valid = s < c.V;  // lanes past the end take part in the barriers on site 0 and store nothing
+        if (!valid) s = 0;
+        int xc[4];
+        site_coords(c, s, xc);
+        const unsigned eb = edge_bits(c, xc);
+        const int Vp = c.Vp;
+        const double* base = w_in + c.w_off;
+        double* xb = acc + c.x_off + (size_t)mu * 8 * Vp;
+        double* cb = clov + c.m_off;
+        fx_guard g;
+        matq<3> sig, kk;  // kk: F - B of a clover plane, from the staple sum before, between and after
+        matx<3> u;
+        Su3Src src{base, Vp};
+        fx_zero(sig);
+        if (MODE != 0) fx_zero(kk);
+        fx_staples<3, true>(sig, src, c, s, mu, eb, g, [&](int nu) { return MODE == 2 && !c_clover_owner[mu][nu]; },
+            [&](int back, int nu, const matq<3>& sum) {
+                if (!valid || MODE == 0) return;
+                if (!c_clover_owner[mu][nu]) {
+                    if (back) kk = sum;
+                    return;
+                }
+                const int pl = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
+                fx_take_matrix<3>(u, src, mu, s, false, g);
+                const long long half = fx_round();
+                if (!back) {
+                    // 3 - Re Tr(U F), the deviation of the twisted plaquette from the unit matrix
+                    long long hh = 0, cr = half;
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) {
+                            int rh, rl, ih, il;
+                            fx_split<1>(sum.re[j][i] - kk.re[j][i], rh, rl);
+                            fx_split<1>(sum.im[j][i] - kk.im[j][i], ih, il);
+                            fx_mad(hh, cr, u.rh[i][j], u.rl[i][j], rh, rl);
+                            fx_mad(hh, cr, fx_neg(u.ih[i][j]), fx_neg(u.il[i][j]), ih, il);
+                            kk.re[j][i] = 2 * sum.re[j][i] - kk.re[j][i];
+                            kk.im[j][i] = 2 * sum.im[j][i] - kk.im[j][i];
+                        }
+                    cb[(size_t)(108 + pl) * Vp + s] = (double)((3ll << 57) - fx_join(hh, cr)) * 0x1p-57;
+                    return;
+                }
+                // K = F - B; D1 = U K (site n), D2 = K U (site n + mu).  A plane built through its second
+                // direction (nu < mu) takes the other sign: its leaves are the conjugates of (mu, nu)'s.
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        kk.re[i][j] -= sum.re[i][j];
+                        kk.im[i][j] -= sum.im[i][j];
+                    }
+                fx_check<3, 28>(kk, g);
+                matx<3> kx;
+                matq<3> t;
+                fx_operand_wide<3, 1>(kx, kk);
+                const double unit = nu > mu ? 0x1p-57 : -0x1p-57;
+                fx_mul_nn<3>(t, u, kx);
+                fx_store_ah(cb + (size_t)(pl * 2 + 0) * 9 * Vp, Vp, s, t, unit);
+                fx_mul_nn<3>(t, kx, u);
+                fx_store_ah(cb + (size_t)(pl * 2 + 1) * 9 * Vp, Vp, fwd(c, eb, s, mu), t, unit);
+                kk = sum;
+            });
+        if (!valid) continue;
+        if (MODE == 2) {
+            if (g.bad()) {
+                alg8<double> z;
+                native_force64<MODE>(z, c, base, cb, s, mu, eb);
+            }
+            continue;
+        }
+        // Omega = U_mu(n) Sigma (units 2^-56), Z = -P_ta(Omega)
+        alg8<double> x, z;
+        {
+            matx<3> sx;
+            matq<3> om;
+            fx_operand_wide<3, 2>(sx, sig);
+            fx_take_matrix<3>(u, src, mu, s, false, g);
+            fx_mul_nn<3>(om, u, sx);
+            const double tr = (double)(om.im[0][0] + om.im[1][1] + om.im[2][2]) * (1.0 / 3.0);
+            z.v[0] = 0x1p-56 * (tr - (double)om.im[0][0]);
+            z.v[1] = 0x1p-56 * (tr - (double)om.im[1][1]);
+            z.v[2] = 0x1p-57 * (double)(om.re[1][0] - om.re[0][1]);
+            z.v[3] = -0x1p-57 * (double)(om.im[0][1] + om.im[1][0]);
+            z.v[4] = 0x1p-57 * (double)(om.re[2][0] - om.re[0][2]);
+            z.v[5] = -0x1p-57 * (double)(om.im[0][2] + om.im[2][0]);
+            z.v[6] = 0x1p-57 * (double)(om.re[2][1] - om.re[1][2]);
+            z.v[7] = -0x1p-57 * (double)(om.im[1][2] + om.im[2][1]);
+        }
+        if (g.bad()) native_force64<MODE>(z, c, base, cb, s, mu, eb);
+        rk3_x<STAGE>(x, z, c.h, xb, Vp, s);
+        mat3<double> e, w;
+        expm_su3<double, true>(e, x);
+        matx<3> ex;
+        const unsigned up = fx_scale_of(e);  // exp(X) - 1 is of the size of the step: scaled up to 1
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) fx_take_entry<3>(ex, i, j, e.e[i][j].re, e.e[i][j].im, g, up);
+        Store<P64>::load(base + (size_t)mu * 18 * Vp, Vp, s, w);
+        // W' = W + (exp(X) - 1) W, the product in fixed point (unless exp(X) - 1 is out of its range),
+        // rounded once onto W
+        if (g.bad()) {
+            mat3<double> d;
+            mul_nn(d, e, w);
+            add_to(w, d);
+        } else {
+            matq<3> d;
+            fx_mul_nn<3>(d, ex, u);
+            const double unit = __hiloint2double((int)((1023u - 58u - up) << 20), 0);  // 2^(-58 - up)
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    w.e[i][j].re = fma((double)d.re[i][j], unit, w.e[i][j].re);
+                    w.e[i][j].im = fma((double)d.im[i][j], unit, w.e[i][j].im);
+                }
+        }
+        Store<P64>::store(w_out + c.w_off + (size_t)mu * 18 * Vp, Vp, s, w);
+    }
+}
+
+}  // namespace tgf

@@ -12,6 +12,7 @@
 
 #include "expm.cuh"
 #include "lattice.cuh"
+#include "planes.cuh"
 
 namespace tgf {
 
@@ -120,25 +121,7 @@ __device__ __forceinline__ void bar_sync(int id, int nthreads) {
 // the measured stage 1 (MODE 1: clover halves too) needs more registers: at most 4 blocks per SM
 template <int P, int TILE, int MODE>
 constexpr int stage_min_blocks() {
-    return P == P64 ? 2 : (MODE != 0 && StageTile<TILE>::minb32 > 4) ? 4 : StageTile<TILE>::minb32;
-}
-
-// Plane index of (mu, nu), mu < nu, in the order 01, 23, 02, 13, 03, 12 (consecutive planes
-// pair up in the topological charge); -1 for mu >= nu.
-static __constant__ int8_t c_plane_of[4][4] = {{-1, 0, 2, 4}, {-1, -1, 5, 3}, {-1, -1, -1, 1}, {-1, -1, -1, -1}};
-static __constant__ int8_t c_pair[6][2] = {{0, 1}, {2, 3}, {0, 2}, {1, 3}, {0, 3}, {1, 2}};
-// Which direction's warp builds the clover halves of each plane: 01, 02 by warp 0; 12, 13 by
-// warp 1; 23 by warp 2; 03 by warp 3 -- two planes at most per warp instead of 3, 2, 1, 0.
-static __constant__ int8_t c_clover_owner[4][4] = {{0, 1, 1, 0}, {0, 0, 1, 1}, {0, 0, 0, 1}, {1, 0, 0, 0}};
-
-// The anti-Hermitian part D - D^+ of a 3x3 matrix as 9 reals (2 Im D_jj; D_jk - conj(D_kj), j<k),
-// written to one slot of the clover scratch (AhStore).
-template <class T>
-__device__ __forceinline__ void store_ah(T* __restrict__ p, int Vp, int s, const mat3<T>& d) {
-    const T v[9] = {T(2) * d.e[0][0].im,           T(2) * d.e[1][1].im,           T(2) * d.e[2][2].im,
-                    d.e[0][1].re - d.e[1][0].re, d.e[0][1].im + d.e[1][0].im, d.e[0][2].re - d.e[2][0].re,
-                    d.e[0][2].im + d.e[2][0].im, d.e[1][2].re - d.e[2][1].re, d.e[1][2].im + d.e[2][1].im};
-    AhStore<T>::store(p, Vp, s, v);
+    return (MODE != 0 && StageTile<TILE>::minb32 > 4) ? 4 : StageTile<TILE>::minb32;
 }
 
 // MODE 0: the RK3 stage.  MODE 1: the stage, and from the same staples of the input field the
@@ -159,21 +142,14 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
     using S = Store<P>;
     constexpr int R = S::reals;
     constexpr int SPB = StageTile<TILE>::spb;
-    static_assert(P != P64 || TILE == 0, "FP64 shares the block's forward-staple corners: tile 0 only");
+    static_assert(P != P64, "FP64: stage64.cuh");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mu = warp & 3;
     const int row = warp >> 2;  // which 32-site row of the block
-    // T_{ab}(n) = U_b(n+a) U_a(n+b)^+ of the six planes a < b: the forward staple of link (n, a) in
-    // direction b is T_ab U_b(n)^+, that of link (n, b) in direction a is T_ab^+ U_a(n)^+, so in
-    // FP64 (bound by the FP64 pipe) each is computed once per site by one warp of the block and
-    // shared behind one block barrier (42 instead of 48 staple products per site).  The FP32 forms,
-    // bound by latency, share them only in launch tile 3, in pairs of warps without a block barrier.
-    constexpr bool SHARE = (P == P64);
-    __shared__ cx<T> sT[SHARE ? 6 : 1][9][32];
     // tile 3 (FP32 forms, unmeasured stages): corners shared in pairs; every lane of the block's four
     // warps takes part in the named barriers, lanes past the configuration's end on site 0 with
     // their results discarded
-    constexpr bool PAIR = (P != P64) && StageTile<TILE>::pair && MODE == 0;
+    constexpr bool PAIR = StageTile<TILE>::pair && MODE == 0;
     __shared__ cx<T> sP[PAIR ? 6 : 1][9][32];
 
     for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
@@ -220,19 +196,6 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
             }
         };
         mat3<T> sig, a, b, t;
-        if constexpr (SHARE) {
-            // phase 1: warp w builds T of planes w and w + 4 (pair order 01, 23, 02, 13, 03, 12)
-            for (int pr = warp; pr < 6; pr += 4) {
-                if (!valid) break;
-                const int pa = c_pair[pr][0], pb = c_pair[pr][1];
-                link(pb, fwd(c, eb, s, pa), a);
-                link(pa, fwd(c, eb, s, pb), b);
-                mul_nd(t, a, b);
-#pragma unroll
-                for (int k = 0; k < 9; ++k) sT[pr][k][lane] = t.e[k / 3][k % 3];
-            }
-            __syncthreads();
-        }
         auto link_body = [&]() {
         const int s_mp = fwd(c, eb, s, mu);
         const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
@@ -251,12 +214,7 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
             const bool tw_f = k != 0 && at_mu0 && ((eb >> nu) & 1u);
             mat3<T> f;
             bool fwd_done = false;  // tile 3: a consumer's shared staple is already in sig
-            if constexpr (SHARE) {
-                // T_{mu nu} = T_{nu mu}^+ from the block's shared T of the plane
-                const int pl_f = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
-#pragma unroll
-                for (int kk = 0; kk < 9; ++kk) t.e[kk / 3][kk % 3] = sT[pl_f][kk][lane];
-            } else if constexpr (PAIR) {
+            if constexpr (PAIR) {
                 const int pl_f = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
                 if (c_pair_own[mu][nu]) {
                     prod_nd(t, nu, s_mp, mu, fwd(c, eb, s, nu), a, b);  // T_{mu nu}
@@ -278,26 +236,15 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
             }
             if (!fwd_done) {
             link(nu, s, a);
-            if (!SHARE || nu > mu) {
-                if (clover) {
-                    mul_nd(f, t, a);
-                    if (tw_f) scale_cx(f, zr, -zi);
-                    if (MODE != 2) add_to(sig, f);
-                } else {
-                    // the centre factor scales T before the accumulating product (Z* T U^+), so a
-                    // twisted corner needs no separate staple matrix
-                    if (tw_f) scale_cx(t, zr, -zi);
-                    mul_nd_acc(sig, t, a);
-                }
-            } else {
-                // F = T_{nu mu}^+ U_nu(n)^+ = (U_nu(n) T_{nu mu})^+
-                mul_nn(b, a, t);
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) f.e[i][j] = {b.e[j][i].re, -b.e[j][i].im};
+            if (clover) {
+                mul_nd(f, t, a);
                 if (tw_f) scale_cx(f, zr, -zi);
-                add_to(sig, f);
+                if (MODE != 2) add_to(sig, f);
+            } else {
+                // the centre factor scales T before the accumulating product (Z* T U^+), so a
+                // twisted corner needs no separate staple matrix
+                if (tw_f) scale_cx(t, zr, -zi);
+                mul_nd_acc(sig, t, a);
             }
             }
             // backward staple B = Z_{mu nu}(n-nu) U_nu(n+mu-nu)^+ U_mu(n-nu)^+ U_nu(n-nu)
@@ -373,12 +320,12 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
         expm_su3<T, true>(b, x);
         if constexpr (TWO_ROW) mul_nn_plus_top(t, b, u, u);  // only rows 0 and 1 are stored
         else mul_nn_plus(t, b, u, u);
-        if (STAGE == 3 && P != P64 && reunit) reunitarize(t);
+        if (STAGE == 3 && reunit) reunitarize(t);
         if (valid) S::store(w_out + c.w_off + (size_t)mu * R * Vp, Vp, s, t);
         };
         if (valid || PAIR) link_body();
-        // sT / sP are rewritten by the next block of the grid-stride loop
-        if constexpr (SHARE || PAIR) __syncthreads();
+        // sP is rewritten by the next block of the grid-stride loop
+        if constexpr (PAIR) __syncthreads();
     }
 }
 

@@ -47,22 +47,22 @@ constexpr int kFxBits = 58;
 
 struct fx_guard {
     unsigned top = 0;   // bit 31: an operand outside its bound
-    unsigned top2 = 0;  // bits 30, 31: a staple sum outside its bound
-    __device__ __forceinline__ bool bad() const { return ((top >> 31) | (top2 >> 30)) != 0; }
+    unsigned top2 = 0;  // not 0: a sum outside its bound
+    __device__ __forceinline__ bool bad() const { return ((top >> 31) | top2) != 0; }
 };
 
 // x -> floor(x 2^58) (negative x: to within one unit, as the bitwise complement of |x|'s image) split
 // into hi, lo.  The mantissa with its leading bit is aligned at the top of 64 bits and
 // shifted right by 1025 - exponent, which leaves x 2^61; shifts past 63 bits give 0.
-// `up` takes x 2^up instead (a matrix of small entries keeps its relative precision).
-__device__ __forceinline__ void fx_take(double x, int& hi, int& lo, fx_guard& g, unsigned up = 0) {
+// `up` takes x 2^up instead (a matrix of small entries keeps its relative precision), flip = -1 takes -x.
+__device__ __forceinline__ void fx_take(double x, int& hi, int& lo, fx_guard& g, unsigned up = 0, int flip = 0) {
     const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
     const unsigned a = h & 0x7fffffffu;
     g.top |= (0x3FF00400u - (up << 20)) - a;  // |x| 2^up <= 1 + 2^-10, else bit 31
     const unsigned s = (1025u - up) - (a >> 20);
     unsigned long long m = ((unsigned long long)(__funnelshift_l(l, h, 11) | 0x80000000u) << 32) | (l << 11);
     asm("shr.b64 %0, %0, %1;" : "+l"(m) : "r"(s));
-    const int sg = (int)h >> 31;
+    const int sg = ((int)h >> 31) ^ flip;
     asm("xor.b32 %0, %1, %2;" : "=r"(hi) : "r"((int)(m >> 32)), "r"(sg));
     asm("shr.u32 %0, %1, 3;" : "=r"(lo) : "r"((unsigned)m ^ (unsigned)sg));
 }
@@ -93,15 +93,15 @@ __device__ __forceinline__ void fx_operand_wide(matx<N>& o, const matq<N>& v) {
             fx_split<SH>(v.im[i][j], o.ih[i][j], o.il[i][j]);
         }
 }
-// |entries| < 8 (B = 29) or 4 (B = 28), else the guard's second word
+// |entries| < 2^(B - 26), else the guard's second word (the top word of a sum counts in 2^-26)
 template <int N, int B>
 __device__ __forceinline__ void fx_check(const matq<N>& v, fx_guard& g) {
-    constexpr int up = 29 - B;
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
         for (int j = 0; j < N; ++j)
-            g.top2 |= (((unsigned)(int)(v.re[i][j] >> 32) + (1u << B)) | ((unsigned)(int)(v.im[i][j] >> 32) + (1u << B))) << up;
+            g.top2 |= (((unsigned)(int)(v.re[i][j] >> 32) + (1u << B)) | ((unsigned)(int)(v.im[i][j] >> 32) + (1u << B))) &
+                      ~((2u << B) - 1u);
 }
 
 // c + a b by one IMAD.WIDE.  Written as C++: mad.wide in PTX becomes a product and a separate 64-bit
@@ -263,8 +263,9 @@ __device__ __forceinline__ void fx_transpose(matq<N>& m) {
         }
 }
 
+// a link, transposed if `tr`; flip = -1 conjugates it
 template <int N, class SRC>
-__device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, int site, bool tr, fx_guard& g) {
+__device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, int site, bool tr, fx_guard& g, int flip = 0) {
     double2 x[N][N];
 #pragma unroll
     for (int i = 0; i < N; ++i)
@@ -273,7 +274,10 @@ __device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, in
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
-        for (int j = 0; j < N; ++j) fx_take_entry<N>(o, i, j, x[i][j].x, x[i][j].y, g);
+        for (int j = 0; j < N; ++j) {
+            fx_take(x[i][j].x, o.rh[i][j], o.rl[i][j], g);
+            fx_take(x[i][j].y, o.ih[i][j], o.il[i][j], g, 0, flip);
+        }
 }
 
 template <int N, bool SYNC, class SRC, class SKIP, class VISIT>
@@ -346,17 +350,20 @@ struct Su3Src {
     static __device__ __forceinline__ void centre(int k, double& zr, double& zi) { tgf::centre<double>(k, zr, zi); }
 };
 
-// The largest up <= 40 for which every entry of m stays below 1 in magnitude times 2^up.
-__device__ __forceinline__ unsigned fx_scale_of(const mat3<double>& m) {
+// The largest up <= 40 for which every entry of m, times 2^up, stays below 1 in magnitude.
+template <int N>
+__device__ __forceinline__ unsigned fx_scale_of(const cx<double> (&m)[N][N]) {
     unsigned a = 0;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < N; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            a = max(a, (unsigned)__double2hiint(m.e[i][j].re) & 0x7fffffffu);
-            a = max(a, (unsigned)__double2hiint(m.e[i][j].im) & 0x7fffffffu);
+        for (int j = 0; j < N; ++j) {
+            a = max(a, (unsigned)__double2hiint(m[i][j].re) & 0x7fffffffu);
+            a = max(a, (unsigned)__double2hiint(m[i][j].im) & 0x7fffffffu);
         }
     return (unsigned)min(max(1022 - (int)(a >> 20), 0), 40);
 }
+// 2^(-58 - up)
+__device__ __forceinline__ double fx_unit(unsigned up) { return __hiloint2double((int)((1023u - kFxBits - up) << 20), 0); }
 
 }  // namespace tgf

@@ -86,19 +86,6 @@ __device__ __forceinline__ void site_coords(const CfgDesc& c, int s, int (&x)[4]
     x[3] = q3;
 }
 
-// The four coordinates packed in 16-bit fields of one 64-bit register, so that a direction
-// chosen at run time costs a shift, not a local-memory array access.
-__device__ __forceinline__ uint64_t pack_coords(const CfgDesc& c, int s) {
-    int x[4];
-    site_coords(c, s, x);
-    return (uint64_t)x[0] | ((uint64_t)x[1] << 16) | ((uint64_t)x[2] << 32) | ((uint64_t)x[3] << 48);
-}
-__device__ __forceinline__ int coord(uint64_t xp, int d) { return (int)((xp >> (16 * d)) & 0xFFFFu); }
-
-// site index of n +- one step along a direction with coordinate x, extent L, stride st (periodic)
-__device__ __forceinline__ int step_p(int s, int x, int L, int st) { return x == L - 1 ? s - (L - 1) * st : s + st; }
-__device__ __forceinline__ int step_m(int s, int x, int L, int st) { return x == 0 ? s + (L - 1) * st : s - st; }
-
 // Boundary flags of a site in one word: bit d  x_d == 0,  bit 4+d  x_d == L_d - 1,  bit 8+d
 // x_d == 1.  With them a neighbour costs a bit test and a select for a direction chosen at run
 // time; the wrap distance (L_d - 1) st_d is st[d+1] - st[d].

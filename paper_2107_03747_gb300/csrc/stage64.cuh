@@ -213,7 +213,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
         mat3<double> e, w;
         expm_su3<double, true>(e, x);
         matx<3> ex;
-        const unsigned up = fx_scale_of(e);  // exp(X) - 1 is of the size of the step: scaled up to 1
+        const unsigned up = fx_scale_of(e.e);  // exp(X) - 1 is of the size of the step: scaled up to 1
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -228,7 +228,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
         } else {
             matq<3> d;
             fx_mul_nn<3>(d, ex, u);
-            const double unit = __hiloint2double((int)((1023u - 58u - up) << 20), 0);  // 2^(-58 - up)
+            const double unit = fx_unit(up);
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll

@@ -7,7 +7,9 @@
 // Luscher's low-storage RK3, W' = exp(X) W, the clover G = -(i/8)(C - C^+), E, q and the twisted
 // plaquette), written for N x N matrices in registers.  The exponential is a Taylor polynomial of
 // degree 7-11 after scaling by 2^-s, evaluated with few products, then squared s times (SU(2):
-// closed form; SU(3): the Cayley-Hamilton form of the SU(3) kernels).
+// closed form; SU(3): the Cayley-Hamilton form of the SU(3) kernels).  Matrix products run in fixed point
+// on the integer pipe (fixed.cuh); the FP64 forms of the products and of the exponential serve links outside
+// its range.
 //
 // Storage per configuration and direction: N^2 double2 planes (matrix entries, row-major) of
 // Vp sites; the RK3 accumulator X holds N^2 reals per link: the imaginary parts of the N
@@ -17,6 +19,7 @@
 #include <stdint.h>
 
 #include "expm.cuh"
+#include "fixed.cuh"
 #include "lattice.cuh"
 
 namespace tgf {
@@ -263,9 +266,224 @@ __device__ void expN<3>(matN<3>& out, const matN<3>& X) {
         for (int j = 0; j < 3; ++j) out.e[i][j] = m.e[i][j];
 }
 
-// one RK3 stage for SU(N); block = 4 warps (one per direction) x 32 sites
+// links for fixed.cuh: entry planes of double2
+template <int N>
+struct SunSrc {
+    const double2* q;
+    int Vp;
+    __device__ __forceinline__ double2 get(int dir, int s, int i, int j, bool tr) const {
+        s = checked_site(s, Vp);
+        return __ldg(q + ((size_t)dir * N * N + (tr ? j * N + i : i * N + j)) * Vp + s);
+    }
+    static __device__ __forceinline__ void centre(int k, double& zr, double& zi) { centreN<N>(k, zr, zi); }
+};
+
+// Omega = U Sigma in FP64, for links whose staples leave the range of fixed.cuh
+template <int N>
+__device__ __forceinline__ void native_omegaN(matN<N>& om, const CfgDesc& c, const double* __restrict__ base, int s, int mu,
+                                              unsigned eb) {
+    const int Vp = c.Vp;
+    const int s_mp = fwd(c, eb, s, mu);
+    const bool at_mu0 = (eb >> mu) & 1u;
+    matN<N> sig, a, b, t;
+    zeroN(sig);
+#pragma unroll 1
+    for (int dn = 1; dn < 4; ++dn) {
+        const int nu = (mu + dn) & 3;
+        const int s_nm = bwd(c, eb, s, nu);
+        const int k = c.tw[mu * 4 + nu];
+        double zr = 1.0, zi = 0.0;
+        if (k != 0) centreN<N>(k, zr, zi);
+        // forward staple Z*_{mu nu}(n) U_nu(n+mu) U_mu(n+nu)^+ U_nu(n)^+
+        loadN<N>(base, Vp, nu, s_mp, a);
+        loadN<N>(base, Vp, mu, fwd(c, eb, s, nu), b);
+        ndN<N, false>(t, a, b);
+        if (k != 0 && at_mu0 && ((eb >> nu) & 1u)) scaleN(t, zr, -zi);
+        loadN<N>(base, Vp, nu, s, a);
+        ndN<N, true>(sig, t, a);
+        // backward staple Z_{mu nu}(n-nu) U_nu(n+mu-nu)^+ U_mu(n-nu)^+ U_nu(n-nu)
+        loadN<N>(base, Vp, mu, s_nm, a);
+        loadN<N>(base, Vp, nu, fwd(c, eb, s_nm, mu), b);
+        nnN<N, false>(t, a, b);
+        if (k != 0 && at_mu0 && ((eb >> (8 + nu)) & 1u)) scaleN(t, zr, -zi);
+        loadN<N>(base, Vp, nu, s_nm, a);
+        dnN<N, true>(sig, t, a);
+    }
+    loadN<N>(base, Vp, mu, s, a);
+    nnN<N, false>(om, a, sig);
+}
+
+// exp(X) - 1 as an operand in units 2^(-58 - up), X traceless anti-Hermitian.  SU(3): the Cayley-Hamilton
+// form of the SU(3) kernels; SU(2): X^2 = -z 1, so exp(X) - 1 = (cos sqrt z - 1) + (sin sqrt z / sqrt z) X, the two
+// functions by their power series in z up to z = 1/4 (the tail of the eighth term is below 1e-18).
+template <int N>
+__device__ __forceinline__ unsigned fx_exp_m1(matx<N>& o, const matN<N>& X, fx_guard& g) {
+    matN<N> m;
+    if constexpr (N == 2) {
+        const double a = 0.5 * (X.e[0][0].im - X.e[1][1].im), br = X.e[0][1].re, bi = X.e[0][1].im;
+        const double z = a * a + br * br + bi * bi;
+        double cm1, sc;
+        if (z <= 0.25) {
+            // 1/k! for k = 2, 4, ... and 1, 3, ...
+            constexpr double f[17] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320,
+                                      1.0 / 362880, 1.0 / 3628800, 1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0,
+                                      1.0 / 87178291200.0, 1.0 / 1307674368000.0, 1.0 / 20922789888000.0};
+            cm1 = f[16];
+            sc = f[15];
+#pragma unroll
+            for (int k = 7; k >= 1; --k) {
+                cm1 = fma(-z, cm1, f[2 * k]);
+                sc = fma(-z, sc, f[2 * k - 1]);
+            }
+            cm1 *= -z;
+        } else {
+            const double th = sqrt(z);
+            double sn, cs;
+            sincos(th, &sn, &cs);
+            cm1 = cs - 1.0;
+            sc = sn / th;
+        }
+        m.e[0][0] = {cm1, sc * a};
+        m.e[1][1] = {cm1, -sc * a};
+        m.e[0][1] = {sc * br, sc * bi};
+        m.e[1][0] = {-sc * br, sc * bi};
+    } else {
+        alg8<double> x;
+        x.v[0] = X.e[0][0].im;
+        x.v[1] = X.e[1][1].im;
+        x.v[2] = X.e[0][1].re;
+        x.v[3] = X.e[0][1].im;
+        x.v[4] = X.e[0][2].re;
+        x.v[5] = X.e[0][2].im;
+        x.v[6] = X.e[1][2].re;
+        x.v[7] = X.e[1][2].im;
+        mat3<double> e;
+        expm_su3<double, true>(e, x);
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) m.e[i][j] = e.e[i][j];
+    }
+    const unsigned up = fx_scale_of(m.e);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) fx_take_entry<N>(o, i, j, m.e[i][j].re, m.e[i][j].im, g, up);
+    return up;
+}
+
+// 1/k! in units 2^-58
+__constant__ long long c_inv_fact[12] = {1ll << 58, 1ll << 58, (1ll << 58) / 2, (1ll << 58) / 6, (1ll << 58) / 24,
+                                         (1ll << 58) / 120, (1ll << 58) / 720, (1ll << 58) / 5040, (1ll << 58) / 40320,
+                                         (1ll << 58) / 362880, (1ll << 58) / 3628800, (1ll << 58) / 39916800};
+
+// SU(4): the Taylor polynomial of expN (same degrees), in fixed point: Y and Y' = 2^up Y as operands, M = Y^2,
+// T = B_1 + M (B_2 + ...) with B_j = 1/(2j)! + Y/(2j+1)!, then exp(Y) - 1 = Y + M T and, s times,
+// exp(2Y) - 1 = 2 (exp(Y) - 1) + (exp(Y) - 1)^2.  M and the last product carry the factor 2^up, so that
+// the small matrix keeps its relative precision.
+template <>
+__device__ __forceinline__ unsigned fx_exp_m1<4>(matx<4>& o, const matN<4>& X, fx_guard& g) {
+    constexpr int N = 4;
+    double n2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = i; j < N; ++j) n2 += (i == j ? 1.0 : 2.0) * (X.e[i][j].re * X.e[i][j].re + X.e[i][j].im * X.e[i][j].im);
+    int s = 0;
+    while (n2 > 0.04 && s < 30) {
+        n2 *= 0.25;
+        ++s;
+    }
+    const int nb = n2 <= 0.028 * 0.028 ? 4 : n2 <= 0.088 * 0.088 ? 5 : 6;
+    const double sc = __hiloint2double((1023 - s) << 20, 0);
+    matN<N> Y;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) Y.e[i][j] = {X.e[i][j].re * sc, X.e[i][j].im * sc};
+    const unsigned up = s > 0 ? 0u : fx_scale_of(Y.e);
+    matx<N> y, m, t;
+    matq<N> q;
+    const long long half = fx_round();
+    {
+        matx<N> yu;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                fx_take_entry<N>(y, i, j, Y.e[i][j].re, Y.e[i][j].im, g);
+                fx_take_entry<N>(yu, i, j, Y.e[i][j].re, Y.e[i][j].im, g, up);
+            }
+        fx_mul_nn<N>(q, y, yu);
+    }
+    // q = 2^up Y^2; m = Y^2
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            fx_split<0>(q.re[i][j] >> up, m.rh[i][j], m.rl[i][j]);
+            fx_split<0>(q.im[i][j] >> up, m.ih[i][j], m.il[i][j]);
+        }
+    matq<N> h;
+    fx_zero(h);
+#pragma unroll 1
+    for (int jb = nb - 1; jb >= 1; --jb) {
+        // h = B_jb + M t (t = 0 for the top block)
+        const long long c0 = c_inv_fact[2 * jb], c1 = c_inv_fact[2 * jb + 1];
+        int c1h, c1l;
+        fx_split<0>(c1, c1h, c1l);
+        const bool top = jb == nb - 1;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const vecx<N> r = fx_row(m, i), nr = fx_negated(r);
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                long long re = i == j ? c0 : 0, im = 0, rc = half, ic = half;
+                fx_mad(re, rc, y.rh[i][j], y.rl[i][j], c1h, c1l);
+                fx_mad(im, ic, y.ih[i][j], y.il[i][j], c1h, c1l);
+                re = fx_join(re, rc);
+                im = fx_join(im, ic);
+                if (!top) fx_dot<N, false>(re, im, r, nr, fx_col(t, j), half);
+                h.re[i][j] = re;
+                h.im[i][j] = im;
+            }
+        }
+        fx_operand_wide<N, 0>(t, h);
+    }
+    // exp(Y) - 1 = Y + M T in units 2^(-58 - up)
+    matx<N> mu_;
+    fx_operand_wide<N, 0>(mu_, q);
+    fx_mul_nn<N>(h, mu_, t);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            h.re[i][j] += (((long long)y.rh[i][j] << 29) + y.rl[i][j]) << up;
+            h.im[i][j] += (((long long)y.ih[i][j] << 29) + y.il[i][j]) << up;
+        }
+    fx_operand_wide<N, 0>(o, h);
+#pragma unroll 1
+    for (int k = 0; k < s; ++k) {
+        fx_mul_nn<N>(q, o, o);
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                h.re[i][j] = 2 * h.re[i][j] + q.re[i][j];
+                h.im[i][j] = 2 * h.im[i][j] + q.im[i][j];
+            }
+        fx_operand_wide<N, 0>(o, h);
+    }
+    fx_check<N, 27>(h, g);
+    return up;
+}
+
+// one RK3 stage for SU(N); block = 4 warps (one per direction) x 32 sites.  Matrix products in fixed point
+// on the integer pipe (fixed.cuh), scalars in FP64, as the SU(3) kernels of stage64.cuh; all of it in FP64 kept
+// that pipe 90-96 % busy.  Two steps and a measurement of 8 x 8x8x16x16 in SU(2): 4.08 ms before, 1.51 now; one
+// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.83 now.
 template <int N, int STAGE, int CAP>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(128, N == 4 ? 2 : 3)
 k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
             double* __restrict__ acc) {
     const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -273,70 +491,64 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
     if (blk >= B.nblk) return;
     const int ci = find_cfg(B, blk);
     const CfgDesc& c = B.c[ci];
-    const int s = (blk - c.blk0) * 32 + lane;
-    if (s >= c.V) return;
-    const uint64_t xp = pack_coords(c, s);
+    int s = (blk - c.blk0) * 32 + lane;
+    const bool valid = s < c.V;  // the others take part in the barriers and store nothing
+    if (!valid) s = 0;
+    int xc[4];
+    site_coords(c, s, xc);
+    const unsigned eb = edge_bits(c, xc);
     const int Vp = c.Vp;
     const double* base = w_in + c.w_off;
-    const int xm = coord(xp, mu), Lm = c.L[mu], Sm = c.st[mu];
-    const int s_mp = step_p(s, xm, Lm, Sm);
-    matN<N> sig, a, b, t;
-    zeroN(sig);
-#pragma unroll 1
-    for (int dn = 1; dn < 4; ++dn) {
-        const int nu = (mu + dn) & 3;
-        const int xn = coord(xp, nu), Ln = c.L[nu], Sn = c.st[nu];
-        const int s_nm = step_m(s, xn, Ln, Sn);
-        const int s_mp_nm = step_p(s_nm, xm, Lm, Sm);
-        const int k = c.tw[mu * 4 + nu];
-        double zr = 1.0, zi = 0.0;
-        if (k != 0) centreN<N>(k, zr, zi);
-        // forward staple Z*_{mu nu}(n) U_nu(n+mu) U_mu(n+nu)^+ U_nu(n)^+
-        loadN<N>(base, Vp, nu, s_mp, a);
-        loadN<N>(base, Vp, mu, step_p(s, xn, Ln, Sn), b);
-        ndN<N, false>(t, a, b);
-        loadN<N>(base, Vp, nu, s, a);
-        if (k != 0 && xm == 0 && xn == 0) {
-            ndN<N, false>(b, t, a);
-            scaleN(b, zr, -zi);
-            addN(sig, b);
-        } else {
-            ndN<N, true>(sig, t, a);
-        }
-        // backward staple Z_{mu nu}(n-nu) U_nu(n+mu-nu)^+ U_mu(n-nu)^+ U_nu(n-nu)
-        loadN<N>(base, Vp, mu, s_nm, a);
-        loadN<N>(base, Vp, nu, s_mp_nm, b);
-        nnN<N, false>(t, a, b);
-        loadN<N>(base, Vp, nu, s_nm, a);
-        if (k != 0 && xm == 0 && xn == 1) {
-            dnN<N, false>(b, t, a);
-            scaleN(b, zr, zi);
-            addN(sig, b);
-        } else {
-            dnN<N, true>(sig, t, a);
-        }
-    }
-    // Omega = U Sigma; Z = -P_ta(Omega) = -(Omega - Omega^+)/2 + tr(Omega - Omega^+)/(2N)
-    loadN<N>(base, Vp, mu, s, a);
-    nnN<N, false>(t, a, sig);
-    double trim = 0.0;
+    fx_guard g;
+    SunSrc<N> src{reinterpret_cast<const double2*>(base), Vp};
+    matx<N> u;
+    matN<N> X;
+    double x[N * N];  // Z, then X: diagonal imaginary parts, then (re, im) above the diagonal
+    {
+        matq<N> sig, om;
+        fx_zero(sig);
+        fx_staples<N, true>(sig, src, c, s, mu, eb, g, [](int) { return false; }, [](int, int, const matq<N>&) {});
+        if (!valid) return;
+        // Omega = U Sigma (units 2^-56); Z = -P_ta(Omega) = -(Omega - Omega^+)/2 + tr(Omega - Omega^+)/(2N)
+        matx<N> sx;
+        fx_operand_wide<N, 2>(sx, sig);
+        fx_take_matrix<N>(u, src, mu, s, false, g);
+        fx_mul_nn<N>(om, u, sx);
+        long long tr = 0;
 #pragma unroll
-    for (int i = 0; i < N; ++i) trim += t.e[i][i].im;
-    trim /= N;
+        for (int i = 0; i < N; ++i) tr += om.im[i][i];
+        const double trim = (double)tr * (1.0 / N);
+        int r = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[r++] = 0x1p-56 * (trim - (double)om.im[i][i]);
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = i + 1; j < N; ++j) {
+                x[r++] = 0x1p-57 * (double)(om.re[j][i] - om.re[i][j]);
+                x[r++] = -0x1p-57 * (double)(om.im[i][j] + om.im[j][i]);
+            }
+    }
+    if (g.bad()) {
+        matN<N> t;
+        native_omegaN<N>(t, c, base, s, mu, eb);
+        double trim = 0.0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) trim += t.e[i][i].im;
+        trim /= N;
+        int r = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[r++] = -(t.e[i][i].im - trim);
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = i + 1; j < N; ++j) {
+                x[r++] = -0.5 * (t.e[i][j].re - t.e[j][i].re);
+                x[r++] = -0.5 * (t.e[i][j].im + t.e[j][i].im);
+            }
+    }
     const double h = c.h;
     double* xb = acc + c.x_off + (size_t)mu * N * N * Vp;
-    // X in N^2 reals: diag imag parts, then (re, im) above the diagonal
-    double x[N * N];
-    int r = 0;
-#pragma unroll
-    for (int i = 0; i < N; ++i) x[r++] = -(t.e[i][i].im - trim);
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-#pragma unroll
-        for (int j = i + 1; j < N; ++j) {
-            x[r++] = -0.5 * (t.e[i][j].re - t.e[j][i].re);
-            x[r++] = -0.5 * (t.e[i][j].im + t.e[j][i].im);
-        }
 #pragma unroll
     for (int q = 0; q < N * N; ++q) {
         double v;
@@ -346,95 +558,146 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
         x[q] = v;
         if (STAGE != 3) xb[(size_t)q * Vp + s] = v;
     }
-    r = 0;
+    int r = 0;
 #pragma unroll
-    for (int i = 0; i < N; ++i) b.e[i][i] = {0.0, x[r++]};
+    for (int i = 0; i < N; ++i) X.e[i][i] = {0.0, x[r++]};
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
         for (int j = i + 1; j < N; ++j) {
-            b.e[i][j] = {x[r], x[r + 1]};
-            b.e[j][i] = {-x[r], x[r + 1]};
+            X.e[i][j] = {x[r], x[r + 1]};
+            X.e[j][i] = {-x[r], x[r + 1]};
             r += 2;
         }
-    expN<N>(t, b);
-    nnN<N, false>(b, t, a);
-    storeN<N>(w_out + c.w_off, Vp, mu, s, b);
+    matx<N> ex;
+    const unsigned up = fx_exp_m1<N>(ex, X, g);
+    matN<N> w;
+    loadN<N>(base, Vp, mu, s, w);
+    if (g.bad()) {
+        matN<N> e, a = w;
+        expN<N>(e, X);
+        nnN<N, false>(w, e, a);
+    } else {
+        // W' = W + (exp(X) - 1) W, rounded once onto W
+        matq<N> d;
+        fx_mul_nn<N>(d, ex, u);
+        const double unit = fx_unit(up);
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                w.e[i][j].re = fma((double)d.re[i][j], unit, w.e[i][j].re);
+                w.e[i][j].im = fma((double)d.im[i][j], unit, w.e[i][j].im);
+            }
+    }
+    storeN<N>(w_out + c.w_off, Vp, mu, s, w);
 }
 
-// G = -(i/8)(C - C^+) of the plane (mu, nu) at site s, from the four twisted leaves (Sec. 3.1, eq. gmunu);
-// also returns Re Tr[Z* P_{mu nu}(n)] (the first leaf)
+// C = sum of the four twisted leaves of the plane (mu, nu) at site s (Sec. 3.1, eq. gmunu), and
+// Re Tr[Z* P_{mu nu}(n)], the first leaf's trace.  Leaf by leaf, a product of four links from the left,
+// each read as it is or as its adjoint, so that one product in a loop serves all twelve:
+//   L1 = Z*(n)       U_mu(n)      U_nu(n+mu)       U_mu(n+nu)^+    U_nu(n)^+
+//   L2 = Z*(n-nu)    U_nu(n-nu)^+ U_mu(n-nu)       U_nu(n-nu+mu)   U_mu(n)^+
+//   L3 = Z*(n-mu)    U_nu(n)      U_mu(n-mu+nu)^+  U_nu(n-mu)^+    U_mu(n-mu)
+//   L4 = Z*(n-mu-nu) U_mu(n-mu)^+ U_nu(n-mu-nu)^+  U_mu(n-mu-nu)   U_nu(n-nu)
+// In bytes of a word, link k of the leaf: bit 0 the direction (0 mu, 1 nu), bit 1 adjoint, bits 2-5 the site of
+// the table below.
+constexpr unsigned leaf_link(int dir, int adj, int site) { return (unsigned)(dir | adj << 1 | site << 2); }
+constexpr unsigned leaf_word(unsigned a, unsigned b, unsigned c, unsigned d) { return a | b << 8 | c << 16 | d << 24; }
+// sites: 0 n, 1 n+mu, 2 n+nu, 3 n-nu, 4 n-nu+mu, 5 n-mu, 6 n-mu+nu, 7 n-mu-nu
+static __constant__ unsigned c_leaf[4] = {
+    leaf_word(leaf_link(0, 0, 0), leaf_link(1, 0, 1), leaf_link(0, 1, 2), leaf_link(1, 1, 0)),
+    leaf_word(leaf_link(1, 1, 3), leaf_link(0, 0, 3), leaf_link(1, 0, 4), leaf_link(0, 1, 0)),
+    leaf_word(leaf_link(1, 0, 0), leaf_link(0, 1, 6), leaf_link(1, 1, 5), leaf_link(0, 0, 5)),
+    leaf_word(leaf_link(0, 1, 5), leaf_link(1, 1, 7), leaf_link(0, 0, 7), leaf_link(1, 0, 3))};
+
+// where the corner of leaf l touches the twisted corner (bits of edge_bits: x = 0 at n, x = 1 one step back)
+__device__ __forceinline__ bool leaf_twisted(unsigned eb, int mu, int nu, int leaf) {
+    return ((eb >> ((leaf & 2 ? 8 : 0) + mu)) & 1u) && ((eb >> ((leaf & 1 ? 8 : 0) + nu)) & 1u);
+}
+__device__ __forceinline__ int leaf_site(const CfgDesc& c, unsigned eb, int s, int mu, int nu, unsigned w) {
+    const int k = (int)(w >> 2) & 15;
+    if (k == 1 || k == 4) s = fwd(c, eb, s, mu);
+    if (k >= 5) s = bwd(c, eb, s, mu);
+    if (k == 2 || k == 6) s = fwd(c, eb, s, nu);
+    if (k == 3 || k == 4 || k == 7) s = bwd(c, eb, s, nu);
+    return s;
+}
+
 template <int N>
-__device__ void cloverN(const CfgDesc& c, const double* __restrict__ base, int s, uint64_t xp, int mu, int nu,
-                        bool traceless, matN<N>& G, double& retr) {
-    const int Vp = c.Vp;
-    const int xm = coord(xp, mu), xn = coord(xp, nu);
-    const int s_mp = step_p(s, xm, c.L[mu], c.st[mu]), s_mm = step_m(s, xm, c.L[mu], c.st[mu]);
-    const int s_np = step_p(s, xn, c.L[nu], c.st[nu]), s_nm = step_m(s, xn, c.L[nu], c.st[nu]);
-    const int s_nm_mp = step_p(s_nm, xm, c.L[mu], c.st[mu]);
-    const int s_mm_np = step_p(s_mm, xn, c.L[nu], c.st[nu]);
-    const int s_mm_nm = step_m(s_mm, xn, c.L[nu], c.st[nu]);
+__device__ __forceinline__ void fx_leaves(matq<N>& C, long long& retr, const SunSrc<N>& src, const CfgDesc& c, int s, unsigned eb,
+                                          int mu, int nu, fx_guard& g) {
+    fx_zero(C);
+    retr = 0;
     const int k = c.tw[mu * 4 + nu];
-    double zr = 1.0, zi = 0.0;
-    if (k != 0) centreN<N>(k, zr, zi);
-    matN<N> C, a, b, t, l;
-    // L1 = Z*(n) U_mu(n) U_nu(n+mu) U_mu(n+nu)^+ U_nu(n)^+
-    loadN<N>(base, Vp, mu, s, a);
-    loadN<N>(base, Vp, nu, s_mp, b);
-    nnN<N, false>(t, a, b);
-    loadN<N>(base, Vp, mu, s_np, a);
-    ndN<N, false>(l, t, a);
-    loadN<N>(base, Vp, nu, s, a);
-    ndN<N, false>(C, l, a);
-    if (k != 0 && xm == 0 && xn == 0) scaleN(C, zr, -zi);
-    retr = 0.0;
-#pragma unroll
-    for (int i = 0; i < N; ++i) retr += C.e[i][i].re;
-    // L2 = Z*(n-nu) U_nu(n-nu)^+ U_mu(n-nu) U_nu(n-nu+mu) U_mu(n)^+
-    loadN<N>(base, Vp, nu, s_nm, a);
-    loadN<N>(base, Vp, mu, s_nm, b);
-    dnN<N, false>(t, a, b);
-    loadN<N>(base, Vp, nu, s_nm_mp, a);
-    nnN<N, false>(l, t, a);
-    loadN<N>(base, Vp, mu, s, a);
-    ndN<N, false>(t, l, a);
-    if (k != 0 && xm == 0 && xn == 1) scaleN(t, zr, -zi);
-    addN(C, t);
-    // L3 = Z*(n-mu) U_nu(n) U_mu(n-mu+nu)^+ U_nu(n-mu)^+ U_mu(n-mu)
-    loadN<N>(base, Vp, nu, s, a);
-    loadN<N>(base, Vp, mu, s_mm_np, b);
-    ndN<N, false>(t, a, b);
-    loadN<N>(base, Vp, nu, s_mm, a);
-    ndN<N, false>(l, t, a);
-    loadN<N>(base, Vp, mu, s_mm, a);
-    nnN<N, false>(t, l, a);
-    if (k != 0 && xm == 1 && xn == 0) scaleN(t, zr, -zi);
-    addN(C, t);
-    // L4 = Z*(n-mu-nu) U_mu(n-mu)^+ U_nu(n-mu-nu)^+ U_mu(n-mu-nu) U_nu(n-nu)
-    loadN<N>(base, Vp, nu, s_mm_nm, b);
-    loadN<N>(base, Vp, mu, s_mm, a);
-    nnN<N, false>(t, b, a);  // U_nu(n-mu-nu) U_mu(n-mu)
-    loadN<N>(base, Vp, mu, s_mm_nm, a);
-    dnN<N, false>(l, t, a);  // (U_nu U_mu)^+ U_mu(n-mu-nu) = U_mu(n-mu)^+ U_nu(n-mu-nu)^+ U_mu(n-mu-nu)
-    loadN<N>(base, Vp, nu, s_nm, a);
-    nnN<N, false>(t, l, a);
-    if (k != 0 && xm == 1 && xn == 1) scaleN(t, zr, -zi);
-    addN(C, t);
-    // G = -(i/8)(C - C^+): G_jk = -(i/8)(C_jk - conj(C_kj))
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const double dr = C.e[i][j].re - C.e[j][i].re, di = C.e[i][j].im + C.e[j][i].im;
-            G.e[i][j] = {di / 8.0, -dr / 8.0};
+#pragma unroll 1
+    for (int leaf = 0; leaf < 4; ++leaf) {
+        unsigned w = c_leaf[leaf];
+        matx<N> t;
+        matq<N> q;
+        fx_take_matrix<N>(t, src, w & 1 ? nu : mu, leaf_site(c, eb, s, mu, nu, w & 0xffu), w & 2, g, w & 2 ? -1 : 0);
+        if (k != 0 && leaf_twisted(eb, mu, nu, leaf)) {
+            double zr, zi;
+            centreN<N>(k, zr, zi);
+            fx_scale(t, zr, -zi);
         }
-    if (traceless) {
-        double tr = 0.0;
+#pragma unroll 1
+        for (int m = 1; m < 4; ++m) {
+            w >>= 8;
+            matx<N> b;
+            fx_take_matrix<N>(b, src, w & 1 ? nu : mu, leaf_site(c, eb, s, mu, nu, w & 0xffu), w & 2, g, w & 2 ? -1 : 0);
+            fx_mul_nn<N>(q, t, b);
+            fx_check<N, 27>(q, g);
+            fx_operand_wide<N, 0>(t, q);
+        }
 #pragma unroll
-        for (int i = 0; i < N; ++i) tr += G.e[i][i].re;
-        tr /= N;
+        for (int i = 0; i < N; ++i) {
+            if (leaf == 0) retr += q.re[i][i];
 #pragma unroll
-        for (int i = 0; i < N; ++i) G.e[i][i].re -= tr;
+            for (int j = 0; j < N; ++j) {
+                C.re[i][j] += q.re[i][j];
+                C.im[i][j] += q.im[i][j];
+            }
+        }
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void native_leaves(matN<N>& C, double& retr, const double* __restrict__ base, const CfgDesc& c, int s,
+                                              unsigned eb, int mu, int nu) {
+    zeroN(C);
+    retr = 0.0;
+    const int k = c.tw[mu * 4 + nu];
+#pragma unroll 1
+    for (int leaf = 0; leaf < 4; ++leaf) {
+        unsigned w = c_leaf[leaf];
+        matN<N> t, b, q;
+        auto take = [&](matN<N>& o) {
+            loadN<N>(base, c.Vp, w & 1 ? nu : mu, leaf_site(c, eb, s, mu, nu, w & 0xffu), q);
+            const bool adj = w & 2;
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    o.e[i][j] = adj ? cx<double>{q.e[j][i].re, -q.e[j][i].im} : q.e[i][j];
+        };
+        take(t);
+        if (k != 0 && leaf_twisted(eb, mu, nu, leaf)) {
+            double zr, zi;
+            centreN<N>(k, zr, zi);
+            scaleN(t, zr, -zi);
+        }
+#pragma unroll 1
+        for (int m = 1; m < 4; ++m) {
+            w >>= 8;
+            take(b);
+            nnN<N, false>(q, t, b);
+            t = q;
+        }
+        if (leaf == 0)
+#pragma unroll
+            for (int i = 0; i < N; ++i) retr += t.e[i][i].re;
+        addN(C, t);
     }
 }
 
@@ -443,9 +706,11 @@ template <int N>
 __device__ __forceinline__ double retr_prod(const matN<N>& A, const matN<N>& B) {
     double v = 0.0;
 #pragma unroll
-    for (int i = 0; i < N; ++i)
+    for (int i = 0; i < N; ++i) {
+        v += A.e[i][i].re * B.e[i][i].re;
 #pragma unroll
-        for (int k = 0; k < N; ++k) v += A.e[i][k].re * B.e[k][i].re - A.e[i][k].im * B.e[k][i].im;
+        for (int k = i + 1; k < N; ++k) v += 2.0 * (A.e[i][k].re * B.e[i][k].re + A.e[i][k].im * B.e[i][k].im);
+    }
     return v;
 }
 
@@ -468,21 +733,55 @@ k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ 
     const int s = (blk - c.blk0) * kSunSites + threadIdx.x;
     double e = 0.0, q = 0.0, p = 0.0, sa = 0.0;
     if (s < c.V) {
-        const uint64_t xp = pack_coords(c, s);
+        int xc[4];
+        site_coords(c, s, xc);
+        const unsigned eb = edge_bits(c, xc);
         const double* base = w + c.w_off;
-        // planes in pairs (01, 23), (02, 13), (03, 12) with the signs of eq. qlatt
-        const int pa[3][2] = {{0, 1}, {0, 2}, {0, 3}}, pb[3][2] = {{2, 3}, {1, 3}, {1, 2}};
-        const double sg[3] = {1.0, -1.0, 1.0};
+        const SunSrc<N> src{reinterpret_cast<const double2*>(base), c.Vp};
+        matN<N> G0;  // the first plane of a pair
 #pragma unroll 1
-        for (int pr = 0; pr < 3; ++pr) {
-            matN<N> Ga, Gb;
-            double ra, rb;
-            cloverN<N>(c, base, s, xp, pa[pr][0], pa[pr][1], traceless, Ga, ra);
-            cloverN<N>(c, base, s, xp, pb[pr][0], pb[pr][1], traceless, Gb, rb);
-            e += retr_prod(Ga, Ga) + retr_prod(Gb, Gb);
-            q += sg[pr] * retr_prod(Ga, Gb);
-            p += (ra + rb) / N;
-            sa += 2.0 * N - (ra + rb);
+        for (int pl = 0; pl < 6; ++pl) {
+            // planes in pairs (01, 23), (02, 13), (03, 12) with the signs of eq. qlatt
+            const int mu = (int)(0x020101u >> (4 * (5 - pl))) & 3, nu = (int)(0x132332u >> (4 * (5 - pl))) & 3;
+            fx_guard g;
+            matN<N> G;
+            double retr, dev;
+            {
+                matq<N> C;
+                long long tr;
+                fx_leaves<N>(C, tr, src, c, s, eb, mu, nu, g);
+                retr = (double)tr * 0x1p-58;
+                dev = (double)(((long long)N << kFxBits) - tr) * 0x1p-58;
+                // G = -(i/8)(C - C^+): G_jk = -(i/8)(C_jk - conj(C_kj))
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+#pragma unroll
+                    for (int j = i; j < N; ++j)
+                        G.e[i][j] = {(double)(C.im[i][j] + C.im[j][i]) * 0x1p-61, -(double)(C.re[i][j] - C.re[j][i]) * 0x1p-61};
+            }
+            if (g.bad()) {
+                matN<N> C;
+                native_leaves<N>(C, retr, base, c, s, eb, mu, nu);
+                dev = N - retr;
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+#pragma unroll
+                    for (int j = i; j < N; ++j)
+                        G.e[i][j] = {(C.e[i][j].im + C.e[j][i].im) / 8.0, -(C.e[i][j].re - C.e[j][i].re) / 8.0};
+            }
+            if (traceless) {
+                double tr = 0.0;
+#pragma unroll
+                for (int i = 0; i < N; ++i) tr += G.e[i][i].re;
+                tr /= N;
+#pragma unroll
+                for (int i = 0; i < N; ++i) G.e[i][i].re -= tr;
+            }
+            e += retr_prod(G, G);
+            if (pl & 1) q += (pl == 3 ? -1.0 : 1.0) * retr_prod(G0, G);
+            else G0 = G;
+            p += retr / N;
+            sa += dev;
         }
         q *= 1.0 / (4.0 * CUDART_PI * CUDART_PI);
     }

@@ -820,16 +820,25 @@ tgf_status tgf_measure_slices(int prec, const tgf_lattice* lat, int ncfg, const 
     Batch H = make_batch(lat, Ly, which, 32);
     launch_stage(prec, 1, 2, 0, H, links, nullptr, nullptr, clover_base(scratch, Ly), st);
     if ((s = last_launch("clover halves"))) return s;
-    // one block per (configuration, slab)
-    Batch Q = make_batch(lat, Ly, which, 1);
-    int blk = 0;
+    // chunks of every slab, and the slabs.  The partial sums fit the scratch's per-block partials (4 doubles per
+    // 128 sites): a slab of k > 1 chunks of 256 has more than 256 (k - 1) >= 128 k sites, and where a
+    // configuration's slabs have one chunk each none are written.
+    Batch Q = make_batch(lat, Ly, which, 1), R = Q;
+    int blk = 0, slab = 0;
+    int64_t off = 0;
     for (int c = 0; c < ncfg; ++c) {
+        const int L = lat[c].L[dir], nch = slice_chunks(Q.c[c].V / L);
         Q.c[c].blk0 = blk;
-        Q.c[c].o_off = c;
-        blk += lat[c].L[dir];
+        R.c[c].blk0 = slab;
+        Q.c[c].o_off = R.c[c].o_off = c;
+        Q.c[c].x_off = R.c[c].x_off = off;
+        blk += L * nch;
+        slab += L;
+        if (nch > 1) off += (int64_t)L * nch;
     }
     Q.nblk = blk;
-    launch_slice_charge(prec, flags, Q, clover_base(scratch, Ly), dir, q_dev, (int)q_stride, st);
+    R.nblk = slab;
+    launch_slice_charge(prec, flags, Q, R, clover_base(scratch, Ly), dir, q_dev, (int)q_stride, scratch, st);
     return last_launch("slice charge");
 }
 

@@ -402,9 +402,12 @@ void launch_reduce(const Batch& B, const double* partial, double* obs, cudaStrea
 // Host: the first observable slot + 1 whose record came out non-finite since the last call (0 if
 // none), read and cleared on `st` (synchronises `st`).
 unsigned long long nonfinite_read_and_clear(cudaStream_t st, cudaError_t* err);
-// per-slab sums of the charge density along `dir`; the batch has L[dir] blocks per configuration
-void launch_slice_charge(int prec, unsigned flags, const Batch& B, const void* clov, int dir, double* q, int q_stride,
-                         cudaStream_t st);
+// Per-slab sums of the charge density along `dir`.  B: L[dir] slice_chunks(V / L[dir]) blocks per configuration, x_off
+// its first partial sum; R: L[dir] blocks per configuration.  partial: a double per block of B.
+constexpr int kSliceSites = 256;
+__host__ __device__ inline int slice_chunks(int n_slab) { return (n_slab + kSliceSites - 1) / kSliceSites; }
+void launch_slice_charge(int prec, unsigned flags, const Batch& B, const Batch& R, const void* clov, int dir, double* q,
+                         int q_stride, double* partial, cudaStream_t st);
 void launch_pack(int prec, const Batch& B, const double* canon, void* w, cudaStream_t st);
 // SU(N) forms (N = 2, 3, 4; FP64): one RK3 stage (batch of 32-site blocks), the measurement
 // (measure batch of 128-site blocks with o_off / h set; partial holds 4 doubles per block), and

@@ -37,6 +37,8 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+constexpr double kSliceUnit = 1.0 / (256.0 * 3.14159265358979323846 * 3.14159265358979323846);
+
 template <class T, int CAP>
 __global__ void __launch_bounds__(kMeasureSites)
 k_clover_sum(const __grid_constant__ BatchT<CAP> B, const T* __restrict__ clov, double* __restrict__ partial,
@@ -149,88 +151,103 @@ k_reduce(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ parti
     }
 }
 
-// q(x0, t) (Sec. 4): the charge density summed over the slab x_dir = x of each configuration,
-// one block per (configuration, slab), FP64 sums in a fixed order.  The launch descriptor has
-// L[dir] blocks per configuration; q_out[cfg_index * q_stride + x] with cfg_index = c.o_off.
+// q(x0, t) (Sec. 4): the charge density summed over the slab x_dir = x of each configuration, FP64 sums in a
+// fixed order.  A slab is cut into chunks of kSliceSites sites, one block and one site per thread each
+// (the launch descriptor has L[dir] slice_chunks(n_slab) blocks per configuration), so that a few long slabs still
+// fill the chip: with one block per slab, 72 slabs of 5184 sites left half the SMs idle and took 75 us, now 29 and 4
+// for the sums (the halves' 161 MB at 6.7 TB/s take 24); tgf_measure_slices of 2 x 12x12x36x36 in FP32 183 -> 139 us.
+// A slab of one chunk is finished here; the
+// others leave a partial sum per block (x_off: the configuration's first one) for k_slice_reduce.
+// q_out[cfg_index * q_stride + x] with cfg_index = c.o_off.
 template <class T, int CAP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSliceSites)
 k_slice_charge(const __grid_constant__ BatchT<CAP> B, const T* __restrict__ clov, int dir, double* __restrict__ q_out,
-               int q_stride, int traceless) {
-    __shared__ double red[256];
-    for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
-        const int ci = find_cfg(B, blk);
-        const CfgDesc& c = B.c[ci];
-        const int x = blk - c.blk0;
-        const int n_slab = c.V / c.L[dir];
+               int q_stride, double* __restrict__ partial, int traceless) {
+    __shared__ double red[kSliceSites / 32];
+    const int ci = find_cfg(B, blockIdx.x);
+    const CfgDesc& c = B.c[ci];
+    const int n_slab = c.V / c.L[dir], nch = slice_chunks(n_slab);
+    const int b = blockIdx.x - c.blk0, x = b / nch, j = (b - x * nch) * kSliceSites + threadIdx.x;
+    double q = 0.0;
+    if (j < n_slab) {
+        // the slab's sites: high st[dir+1] + x st[dir] + low with j = high st[dir] + low
+        const int st = c.st[dir], high = j / st;
+        const int s = high * c.st[dir + 1] + x * st + (j - high * st);
         const T* cb = clov + c.m_off;
         const size_t Vp = (size_t)c.Vp;
-        double acc = 0.0;
-        for (int j = threadIdx.x; j < n_slab; j += 256) {
-            int r = j, s = x * c.st[dir];
+        T a0[9], tq = T(0);
 #pragma unroll
-            for (int d = 0; d < 4; ++d) {
-                if (d == dir) continue;
-                s += (r % c.L[d]) * c.st[d];
-                r /= c.L[d];
+        for (int p = 0; p < 6; ++p) {
+            T a[9], a1[9];
+            AhStore<T>::load(cb + (size_t)(p * 2) * 9 * Vp, (int)Vp, s, a);
+            AhStore<T>::load(cb + (size_t)(p * 2 + 1) * 9 * Vp, (int)Vp, s, a1);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) a[k] += a1[k];
+            if (traceless) {
+                const T tr = (a[0] + a[1] + a[2]) * (T(1) / T(3));
+                a[0] -= tr; a[1] -= tr; a[2] -= tr;
             }
-            T a0[9], tq = T(0);
+            if (p & 1) {
+                const T d = a0[0] * a[0] + a0[1] * a[1] + a0[2] * a[2] +
+                            T(2) * (a0[3] * a[3] + a0[4] * a[4] + a0[5] * a[5] + a0[6] * a[6] + a0[7] * a[7] + a0[8] * a[8]);
+                tq += (p == 3) ? -d : d;
+            } else {
 #pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                T a[9], a1[9];
-                AhStore<T>::load(cb + (size_t)(p * 2) * 9 * Vp, (int)Vp, s, a);
-                AhStore<T>::load(cb + (size_t)(p * 2 + 1) * 9 * Vp, (int)Vp, s, a1);
-#pragma unroll
-                for (int k = 0; k < 9; ++k) a[k] += a1[k];
-                if (traceless) {
-                    const T tr = (a[0] + a[1] + a[2]) * (T(1) / T(3));
-                    a[0] -= tr; a[1] -= tr; a[2] -= tr;
-                }
-                if (p & 1) {
-                    const T d = a0[0] * a[0] + a0[1] * a[1] + a0[2] * a[2] +
-                                T(2) * (a0[3] * a[3] + a0[4] * a[4] + a0[5] * a[5] + a0[6] * a[6] + a0[7] * a[7] + a0[8] * a[8]);
-                    tq += (p == 3) ? -d : d;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 9; ++k) a0[k] = a[k];
-                }
+                for (int k = 0; k < 9; ++k) a0[k] = a[k];
             }
-            acc += (double)tq;
         }
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            const double pi = 3.14159265358979323846;
-            q_out[(size_t)c.o_off * q_stride + x] = red[0] / (256.0 * pi * pi);
-        }
-        __syncthreads();
+        q = (double)tq;
     }
+    q = warp_sum(q);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = q;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+#pragma unroll
+        for (int i = 0; i < kSliceSites / 32; ++i) v += red[i];
+        if (nch == 1) q_out[(size_t)c.o_off * q_stride + x] = v * kSliceUnit;
+        else partial[c.x_off + b] = v;
+    }
+}
+
+// One warp per slab of more than one chunk: its partial sums in a fixed order (blocks: L[dir] per configuration).
+template <int CAP>
+__global__ void __launch_bounds__(32)
+k_slice_reduce(const __grid_constant__ BatchT<CAP> B, int dir, double* __restrict__ q_out, int q_stride,
+               const double* __restrict__ partial) {
+    const int ci = find_cfg(B, blockIdx.x);
+    const CfgDesc& c = B.c[ci];
+    const int nch = slice_chunks(c.V / c.L[dir]);
+    if (nch == 1) return;
+    const int x = blockIdx.x - c.blk0;
+    double v = 0.0;
+    for (int i = threadIdx.x; i < nch; i += 32) v += partial[c.x_off + (int64_t)x * nch + i];
+    v = warp_sum(v);
+    if (threadIdx.x == 0) q_out[(size_t)c.o_off * q_stride + x] = v * kSliceUnit;
 }
 
 template <class T, int CAP>
-static void slices_cap(const Batch& B, const void* clov, int dir, double* q, int q_stride, unsigned flags,
-                       cudaStream_t st) {
-    if constexpr (CAP == kMaxCfg) {
-        k_slice_charge<T, kMaxCfg><<<B.nblk, 256, 0, st>>>(B, (const T*)clov, dir, q, q_stride, (int)(flags & 1u));
-    } else {
-        BatchT<CAP> b;
-        b.ncfg = B.ncfg;
-        b.nblk = B.nblk;
-        for (int i = 0; i < B.ncfg; ++i) b.c[i] = B.c[i];
-        k_slice_charge<T, CAP><<<B.nblk, 256, 0, st>>>(b, (const T*)clov, dir, q, q_stride, (int)(flags & 1u));
+static void slices_cap(const Batch& B, const Batch& R, const void* clov, int dir, double* q, int q_stride, double* partial,
+                       unsigned flags, cudaStream_t st) {
+    BatchT<CAP> b, r;
+    b.ncfg = r.ncfg = B.ncfg;
+    b.nblk = B.nblk;
+    r.nblk = R.nblk;
+    for (int i = 0; i < B.ncfg; ++i) {
+        b.c[i] = B.c[i];
+        r.c[i] = R.c[i];
     }
+    k_slice_charge<T, CAP><<<b.nblk, kSliceSites, 0, st>>>(b, (const T*)clov, dir, q, q_stride, partial, (int)(flags & 1u));
+    if (b.nblk > r.nblk) k_slice_reduce<CAP><<<r.nblk, 32, 0, st>>>(r, dir, q, q_stride, partial);
 }
 
-void launch_slice_charge(int prec, unsigned flags, const Batch& B, const void* clov, int dir, double* q, int q_stride,
-                         cudaStream_t st) {
+void launch_slice_charge(int prec, unsigned flags, const Batch& B, const Batch& R, const void* clov, int dir, double* q,
+                         int q_stride, double* partial, cudaStream_t st) {
     const bool small = B.ncfg <= kSmallCap;
-    if (prec == P64) small ? slices_cap<double, kSmallCap>(B, clov, dir, q, q_stride, flags, st)
-                           : slices_cap<double, kMaxCfg>(B, clov, dir, q, q_stride, flags, st);
-    else small ? slices_cap<float, kSmallCap>(B, clov, dir, q, q_stride, flags, st)
-               : slices_cap<float, kMaxCfg>(B, clov, dir, q, q_stride, flags, st);
+    if (prec == P64) small ? slices_cap<double, kSmallCap>(B, R, clov, dir, q, q_stride, partial, flags, st)
+                           : slices_cap<double, kMaxCfg>(B, R, clov, dir, q, q_stride, partial, flags, st);
+    else small ? slices_cap<float, kSmallCap>(B, R, clov, dir, q, q_stride, partial, flags, st)
+               : slices_cap<float, kMaxCfg>(B, R, clov, dir, q, q_stride, partial, flags, st);
 }
 
 template <class T, int CAP>

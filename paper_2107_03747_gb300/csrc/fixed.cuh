@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "expm.cuh"
 #include "lattice.cuh"
 #include "su3.cuh"
 
@@ -248,7 +249,8 @@ __device__ __forceinline__ void fx_take_entry(matx<N>& o, int i, int j, double r
 // fetch the same instructions at the same time: 11 % on the FP64 stage (8.63 instead of 9.74 ms for
 // 4 steps of 4 x 8x8x24x24).
 // visit(q, nu, sig): called after the forward (q = 0) and after the backward staple (q = 1) of a direction,
-// with the sum in normal orientation; skip(nu) leaves a direction out.
+// with the sum in normal orientation; skip(nu) leaves a direction out.  q0, q1: the part of the six staples (in
+// pairs) that this thread sums.
 template <int N>
 __device__ __forceinline__ void fx_transpose(matq<N>& m) {
 #pragma unroll
@@ -282,12 +284,12 @@ __device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, in
 
 template <int N, bool SYNC, class SRC, class SKIP, class VISIT>
 __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const CfgDesc& c, int s, int mu, unsigned eb, fx_guard& g,
-                                           SKIP&& skip, VISIT&& visit) {
+                                           SKIP&& skip, VISIT&& visit, int q0 = 0, int q1 = 6) {
     const int s_mp = fwd(c, eb, s, mu);
     const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
     const long long half = fx_round();
 #pragma unroll 1
-    for (int q = 0; q < 6; ++q) {
+    for (int q = q0; q < q1; ++q) {
         const bool back = q & 1;
         const int nu = (mu + 1 + (q >> 1)) & 3;
         if (SYNC) __syncthreads();
@@ -365,5 +367,136 @@ __device__ __forceinline__ unsigned fx_scale_of(const cx<double> (&m)[N][N]) {
 }
 // 2^(-58 - up)
 __device__ __forceinline__ double fx_unit(unsigned up) { return __hiloint2double((int)((1023u - kFxBits - up) << 20), 0); }
+
+// ---- exp(X) - 1 of a traceless anti-Hermitian 3x3 matrix ------------------------------------------
+//
+// For X = iQ with ||Q||_F^2 <= kFxExpMax: exp(iQ) - 1 = f0 + f1 Q + f2 Q^2 (f0 without its 1) with the f as the sums
+// over n <= 10 of i^n/n! times the coefficients of Q^n (expm.cuh's recursion, written out as polynomials in
+// c1 = tr Q^2 / 2 and c0 = tr Q^3 / 3); the dropped tail is below 0.126^11 / 11! = 3e-18.  Q is scaled by 2^up to the
+// size of 1, Q^2, the traces and the assembly run in fixed point, the 6 polynomials in FP64: about 45 FP64
+// instructions where the series of expm_su3 takes 210, each of which holds the pipe for 64 cycles and drags four
+// empty issue slots behind it.  Result: operands in units 2^(-58 - up); false if ||Q||_F is too large.
+constexpr double kFxExpMax = 0.016;
+
+struct fx_num {
+    int h, l;
+};
+__device__ __forceinline__ void fx_mac(long long& hh, long long& cr, const fx_num& a, const fx_num& b) {
+    fx_mad(hh, cr, a.h, a.l, b.h, b.l);
+}
+__device__ __forceinline__ fx_num fx_minus(const fx_num& a) { return {fx_neg(a.h), fx_neg(a.l)}; }
+__device__ __forceinline__ fx_num fx_operand(long long v) {
+    fx_num o;
+    fx_split<0>(v, o.h, o.l);
+    return o;
+}
+__device__ __forceinline__ fx_num fx_number(double x, fx_guard& g, unsigned up, int flip = 0) {
+    fx_num o;
+    fx_take(x, o.h, o.l, g, up, flip);
+    return o;
+}
+// s + a b + c d
+__device__ __forceinline__ long long fx_sum2(long long s, const fx_num& a, const fx_num& b, const fx_num& c, const fx_num& d,
+                                             long long half) {
+    long long cr = half;
+    fx_mac(s, cr, a, b);
+    fx_mac(s, cr, c, d);
+    return fx_join(s, cr);
+}
+
+__device__ __forceinline__ bool fx_exp_su3(matx<3>& o, unsigned& up, const alg8<double>& x) {
+    fx_guard g;
+    const long long half = fx_round();
+    const double x22 = -(x.v[0] + x.v[1]);
+    unsigned amax = (unsigned)__double2hiint(x22) & 0x7fffffffu;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) amax = max(amax, (unsigned)__double2hiint(x.v[i]) & 0x7fffffffu);
+    up = (unsigned)min(max(1022 - (int)(amax >> 20), 0), 40);
+    // Q = -i X, times 2^up
+    const fx_num a[3] = {fx_number(x.v[0], g, up), fx_number(x.v[1], g, up), fx_number(x22, g, up)};
+    const fx_num qr[3] = {fx_number(x.v[3], g, up), fx_number(x.v[5], g, up), fx_number(x.v[7], g, up)};  // 01, 02, 12
+    const fx_num qi[3] = {fx_number(x.v[2], g, up, -1), fx_number(x.v[4], g, up, -1), fx_number(x.v[6], g, up, -1)};
+    // Q^2, times 2^(2 up)
+    long long n[3], d[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        n[i] = fx_sum2(0, qr[i], qr[i], qi[i], qi[i], half);
+        long long cr = half;
+        d[i] = 0;
+        fx_mac(d[i], cr, a[i], a[i]);
+        d[i] = fx_join(d[i], cr);
+    }
+    d[0] += n[0] + n[1];
+    d[1] += n[0] + n[2];
+    d[2] += n[1] + n[2];
+    const double two_up = fx_unit(2 * up);
+    const double c1 = 0.5 * two_up * (double)(d[0] + d[1] + d[2]);
+    // u01 = -a2 q01 + q02 q12^*, u02 = -a1 q02 + q01 q12, u12 = -a0 q12 + q01^* q02
+    long long ur[3], ui[3];
+    {
+        const fx_num ma0 = fx_minus(a[0]), ma1 = fx_minus(a[1]), ma2 = fx_minus(a[2]);
+        const fx_num mi12 = fx_minus(qi[2]), mi01 = fx_minus(qi[0]);
+        ur[0] = fx_sum2(fx_sum2(0, ma2, qr[0], qr[1], qr[2], half), qi[1], qi[2], {0, 0}, {0, 0}, half);
+        ui[0] = fx_sum2(fx_sum2(0, ma2, qi[0], qi[1], qr[2], half), qr[1], mi12, {0, 0}, {0, 0}, half);
+        ur[1] = fx_sum2(fx_sum2(0, ma1, qr[1], qr[0], qr[2], half), qi[0], mi12, {0, 0}, {0, 0}, half);
+        ui[1] = fx_sum2(fx_sum2(0, ma1, qi[1], qr[0], qi[2], half), qi[0], qr[2], {0, 0}, {0, 0}, half);
+        ur[2] = fx_sum2(fx_sum2(0, ma0, qr[2], qr[0], qr[1], half), qi[0], qi[1], {0, 0}, {0, 0}, half);
+        ui[2] = fx_sum2(fx_sum2(0, ma0, qi[2], qr[0], qi[1], half), mi01, qr[1], {0, 0}, {0, 0}, half);
+    }
+    // Q^2 times 2^up as operands, and c0 = tr Q^3 / 3
+    fx_num dx[3], vr[3], vi[3];
+    long long t = 0, tc = half, t2 = 0, t2c = half;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        dx[i] = fx_operand(d[i] >> up);
+        vr[i] = fx_operand(ur[i] >> up);
+        vi[i] = fx_operand(ui[i] >> up);
+        fx_mac(t, tc, a[i], dx[i]);
+        fx_mac(t2, t2c, qr[i], vr[i]);
+        fx_mac(t2, t2c, qi[i], vi[i]);
+    }
+    const double c0 = two_up * (1.0 / 3.0) * (double)(fx_join(t, tc) + 2 * fx_join(t2, t2c));
+    const double w = c0 * c0, c2 = c1 * c1;
+    const double a3 = fma(c1, c2, w), a4 = fma(c1, a3, 2.0 * w * c1);
+    const double f2r = fma(a4, -1.0 / 3628800, fma(a3, 1.0 / 40320, fma(c2, -1.0 / 720, fma(c1, 1.0 / 24, -0.5))));
+    const double f2i = c0 * fma(c2, 3.0 / 362880, fma(c1, -2.0 / 5040, 1.0 / 120));
+    const double f1i = fma(a4, 1.0 / 362880, fma(a3, -1.0 / 5040, fma(c2, 1.0 / 120, fma(c1, -1.0 / 6, 1.0))));
+    const double f1r = c0 * fma(fma(4.0 * c1, c2, w), -1.0 / 3628800, fma(c2, 3.0 / 40320, fma(c1, -2.0 / 720, 1.0 / 24)));
+    const double f0r = w * fma(c2, -3.0 / 3628800, fma(c1, 2.0 / 40320, -1.0 / 720));
+    const double f0i = c0 * fma(a3, 1.0 / 362880, fma(c2, -1.0 / 5040, fma(c1, 1.0 / 120, -1.0 / 6)));
+    const fx_num g1r = fx_number(f1r, g, 0), g1i = fx_number(f1i, g, 0), g2r = fx_number(f2r, g, 0), g2i = fx_number(f2i, g, 0);
+    const fx_num g0r = fx_number(f0r, g, up), g0i = fx_number(f0i, g, up);
+    const long long f0re = ((long long)g0r.h << 29) + g0r.l, f0im = ((long long)g0i.h << 29) + g0i.l;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        fx_split<0>(fx_sum2(f0re, g1r, a[i], g2r, dx[i], half), o.rh[i][i], o.rl[i][i]);
+        fx_split<0>(fx_sum2(f0im, g1i, a[i], g2i, dx[i], half), o.ih[i][i], o.il[i][i]);
+        // off-diagonal pair: with A, D = f1 re q + f2 re u and C, B = f1 im q + f2 im u, m_ij = (A - B, D + C),
+        // m_ji = (A + B, D - C)
+        const int p = i == 2 ? 1 : 0, q = i == 0 ? 1 : 2;
+        const long long A = fx_sum2(0, g1r, qr[i], g2r, vr[i], half), D = fx_sum2(0, g1i, qr[i], g2i, vr[i], half);
+        const long long C = fx_sum2(0, g1r, qi[i], g2r, vi[i], half), Bv = fx_sum2(0, g1i, qi[i], g2i, vi[i], half);
+        fx_split<0>(A - Bv, o.rh[p][q], o.rl[p][q]);
+        fx_split<0>(D + C, o.ih[p][q], o.il[p][q]);
+        fx_split<0>(A + Bv, o.rh[q][p], o.rl[q][p]);
+        fx_split<0>(D - C, o.ih[q][p], o.il[q][p]);
+    }
+    return !g.bad() && 2.0 * c1 <= kFxExpMax;
+}
+
+// exp(X) - 1 as operands in units 2^(-58 - up): the form above, or, for larger X and where the caller needs it in
+// FP64 (`general`), the series of expm_su3
+__device__ __forceinline__ unsigned fx_exp_m1_su3(matx<3>& o, mat3<double>& e, const alg8<double>& x, bool general, fx_guard& g) {
+    unsigned up;
+    if (!fx_exp_su3(o, up, x) || general) {
+        expm_su3<double, true>(e, x);
+        up = fx_scale_of(e.e);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) fx_take_entry<3>(o, i, j, e.e[i][j].re, e.e[i][j].im, g, up);
+    }
+    return up;
+}
 
 }  // namespace tgf

@@ -1,13 +1,13 @@
 // stage64.cuh -- one RK3 stage, the clover halves, or both, in double precision: links, the accumulator
-// X and the exponential in FP64, the matrix products in 58-bit fixed point on the integer pipe
-// (fixed.cuh).
+// X and scalars in FP64, the matrix products and the exponential's assembly in 58-bit fixed point on the
+// integer pipe (fixed.cuh).
 //
-// With every product in FP64 the stage kept the FP64 pipe 94-97 % busy (107,000 cycles per warp and SM
-// quarter), and nothing else of the chip was in use.  Here that pipe carries the exponential and the
-// conversions (about 290 instructions, 19,000 cycles), the integer pipe 13 products (4,700 IMAD.WIDE
-// of 4 cycles) and the splitting of the operands, side by side: 36,000 cycles.  4 steps of
-// 4 x 8x8x24x24, measured each step: 23.7 ms before, 8.6 now; one measurement of 4 x 7x7x21x21: 693 us
-// before, 312 now; 3 steps of 4x4x12x12 (latency): 696 us before, 392 now.
+// With everything in FP64 the stage kept the FP64 pipe 94-97 % busy (107,000 cycles per warp and SM
+// quarter), and nothing else of the chip was in use.  Here that pipe carries about 115 instructions (7,200
+// cycles) and the integer pipe 13 products (4,900 IMAD.WIDE of 4 cycles) and the splitting of the operands:
+// 34,000 cycles, the multiply pipe 65 % busy.  4 steps of 4 x 8x8x24x24, measured each step: 23.8 ms before,
+// 8.6 with the products in fixed point, 7.8 with the exponential (fx_exp_su3) as well; one measurement of
+// 4 x 7x7x21x21: 693 us before, 312 now; 3 steps of 4x4x12x12 (latency): 698 us before, 295 now.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -48,7 +48,7 @@ __device__ __forceinline__ void rk3_x(alg8<double>& x, const alg8<double>& z, do
 // fixed.cuh (entries above 1 + 2^-10, infinities, NaN): any input, at the FP64 pipe's rate.
 template <int MODE>
 __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c, const double* __restrict__ base,
-                                               double* __restrict__ cb, int s, int mu, unsigned eb) {
+                                               double* __restrict__ cb, int s, int mu, unsigned eb, int dn0 = 1, int dn1 = 4) {
     const int Vp = c.Vp;
     auto link = [&](int dir, int site, mat3<double>& u) { Store<P64>::load(base + (size_t)dir * 18 * Vp, Vp, site, u); };
     mat3<double> sig, a, b, t, f;
@@ -56,7 +56,7 @@ __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c
     const int s_mp = fwd(c, eb, s, mu);
     const bool at_mu0 = (eb >> mu) & 1u;
 #pragma unroll 1
-    for (int dn = 1; dn < 4; ++dn) {
+    for (int dn = dn0; dn < dn1; ++dn) {
         const int nu = (mu + dn) & 3;
         const bool clover = MODE != 0 && c_clover_owner[mu][nu];
         if (MODE == 2 && !clover) continue;
@@ -110,11 +110,17 @@ __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c
 
 // One thread per link; a block covers 32 sites x 4 directions, warps grouped by mu.  MODE as in k_stage:
 // 0 the stage, 1 the stage and the clover halves of the input field, 2 the halves only.
-template <int STAGE, int MODE, int CAP>
-__global__ void __launch_bounds__(128, MODE == 0 ? 3 : 2)
+//
+// WIDE: three threads per link, one for each direction nu, whose staple sums meet in shared memory (whole numbers:
+// the result is the same to the bit) before the first goes on with the link.  For launches that leave most of
+// the chip idle (launch_m in stage64.cu).
+template <int STAGE, int MODE, int CAP, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 384 : 128, WIDE ? 1 : MODE == 0 ? 3 : 2)
 k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
           double* __restrict__ acc, double* __restrict__ clov) {
-    const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int mu = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31, part = threadIdx.x >> 7;
+    __shared__ long long s_sum[WIDE && MODE != 2 ? 2 : 1][WIDE && MODE != 2 ? 18 : 1][128];
+    __shared__ unsigned s_bad[2][128];
     for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
         const int ci = find_cfg(B, blk);
         const CfgDesc& c = B.c[ci];
@@ -181,12 +187,37 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 fx_mul_nn<3>(t, kx, u);
                 fx_store_ah(cb + (size_t)(pl * 2 + 1) * 9 * Vp, Vp, fwd(c, eb, s, mu), t, unit);
                 kk = sum;
-            });
+            },
+            WIDE ? 2 * part : 0, WIDE ? 2 * part + 2 : 6);
+        if constexpr (WIDE && MODE != 2) {
+            const int lt = threadIdx.x & 127;
+            __syncthreads();  // the block before has read its sums
+            if (part) {
+                s_bad[part - 1][lt] = g.bad();
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    s_sum[part - 1][i][lt] = sig.re[i / 3][i % 3];
+                    s_sum[part - 1][9 + i][lt] = sig.im[i / 3][i % 3];
+                }
+            }
+            __syncthreads();
+            if (part) continue;
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                g.top2 |= s_bad[p][lt];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    sig.re[i / 3][i % 3] += s_sum[p][i][lt];
+                    sig.im[i / 3][i % 3] += s_sum[p][9 + i][lt];
+                }
+            }
+            fx_check<3, 29>(sig, g);
+        }
         if (!valid) continue;
         if (MODE == 2) {
             if (g.bad()) {
                 alg8<double> z;
-                native_force64<MODE>(z, c, base, cb, s, mu, eb);
+                native_force64<MODE>(z, c, base, cb, s, mu, eb, WIDE ? 1 + part : 1, WIDE ? 2 + part : 4);
             }
             continue;
         }
@@ -211,15 +242,10 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
         if (g.bad()) native_force64<MODE>(z, c, base, cb, s, mu, eb);
         rk3_x<STAGE>(x, z, c.h, xb, Vp, s);
         mat3<double> e, w;
-        expm_su3<double, true>(e, x);
         matx<3> ex;
-        const unsigned up = fx_scale_of(e.e);  // exp(X) - 1 is of the size of the step: scaled up to 1
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) fx_take_entry<3>(ex, i, j, e.e[i][j].re, e.e[i][j].im, g, up);
+        const unsigned up = fx_exp_m1_su3(ex, e, x, g.bad(), g);
         Store<P64>::load(base + (size_t)mu * 18 * Vp, Vp, s, w);
-        // W' = W + (exp(X) - 1) W, the product in fixed point (unless exp(X) - 1 is out of its range),
+        // W' = W + (exp(X) - 1) W, the product in fixed point (unless a factor is out of its range),
         // rounded once onto W
         if (g.bad()) {
             mat3<double> d;

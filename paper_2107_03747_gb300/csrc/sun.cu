@@ -313,11 +313,17 @@ __device__ __forceinline__ void native_omegaN(matN<N>& om, const CfgDesc& c, con
     nnN<N, false>(om, a, sig);
 }
 
-// exp(X) - 1 as an operand in units 2^(-58 - up), X traceless anti-Hermitian.  SU(3): the Cayley-Hamilton
-// form of the SU(3) kernels; SU(2): X^2 = -z 1, so exp(X) - 1 = (cos sqrt z - 1) + (sin sqrt z / sqrt z) X, the two
+// exp(X) - 1 as an operand in units 2^(-58 - up), X traceless anti-Hermitian.  SU(3): fx_exp_m1_su3; SU(2):
+// X^2 = -z 1, so exp(X) - 1 = (cos sqrt z - 1) + (sin sqrt z / sqrt z) X, the two
 // functions by their power series in z up to z = 1/4 (the tail of the eighth term is below 1e-18).
 template <int N>
 __device__ __forceinline__ unsigned fx_exp_m1(matx<N>& o, const matN<N>& X, fx_guard& g) {
+    if constexpr (N == 3) {
+        const alg8<double> x = {{X.e[0][0].im, X.e[1][1].im, X.e[0][1].re, X.e[0][1].im, X.e[0][2].re, X.e[0][2].im,
+                                 X.e[1][2].re, X.e[1][2].im}};
+        mat3<double> e;
+        return fx_exp_m1_su3(o, e, x, false, g);
+    }
     matN<N> m;
     if constexpr (N == 2) {
         const double a = 0.5 * (X.e[0][0].im - X.e[1][1].im), br = X.e[0][1].re, bi = X.e[0][1].im;
@@ -347,22 +353,6 @@ __device__ __forceinline__ unsigned fx_exp_m1(matx<N>& o, const matN<N>& X, fx_g
         m.e[1][1] = {cm1, -sc * a};
         m.e[0][1] = {sc * br, sc * bi};
         m.e[1][0] = {-sc * br, sc * bi};
-    } else {
-        alg8<double> x;
-        x.v[0] = X.e[0][0].im;
-        x.v[1] = X.e[1][1].im;
-        x.v[2] = X.e[0][1].re;
-        x.v[3] = X.e[0][1].im;
-        x.v[4] = X.e[0][2].re;
-        x.v[5] = X.e[0][2].im;
-        x.v[6] = X.e[1][2].re;
-        x.v[7] = X.e[1][2].im;
-        mat3<double> e;
-        expm_su3<double, true>(e, x);
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-#pragma unroll
-            for (int j = 0; j < N; ++j) m.e[i][j] = e.e[i][j];
     }
     const unsigned up = fx_scale_of(m.e);
 #pragma unroll

@@ -9,42 +9,71 @@
 
 namespace tgf {
 
+// Both kernels are bound by HBM: a site takes 576 canonical bytes and 192-576 stored ones.  The canonical field is read
+// and written in its own order, consecutive threads on consecutive doubles, and the links change hands in
+// shared memory, a site per row of 73 (odd: the rows of a warp's lanes start in different banks).  A thread that
+// moved its link's 18 doubles itself touched 32 sectors per store, 8 bytes of each: 4 x 16x16x48x48 in FP32
+// packed in 403 us and unpacked in 1185 us (2.04 GB each, 306 us at 6.67 TB/s); now 283 and 311.
+constexpr int kRow = 73;
+
+// float -> double.  The FP64 pipe converts 1.9 lanes per clock and SM (294 us for the 170 million entries of
+// that field); a normal number widens by three shifts of its bits, which the integer pipe has to spare.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x);
+    if (((u + 0x00800000u) & 0x7f000000u) == 0) return (double)x;  // 0, subnormal, infinite or NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 template <int P, int CAP>
 __global__ void __launch_bounds__(128)
 k_pack(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ canon, typename Store<P>::T* __restrict__ w) {
     using T = typename Store<P>::T;
-    for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
-        const int ci = find_cfg(B, blk);
-        const CfgDesc& c = B.c[ci];
-        const int mu = threadIdx.x >> 5;
-        const int s = (blk - c.blk0) * 32 + (threadIdx.x & 31);
-        if (s >= c.V) continue;
-        const double* src = canon + c.x_off + ((size_t)s * 4 + mu) * 18;
-        mat3<T> u;
+    __shared__ T buf[32 * kRow];
+    const int ci = find_cfg(B, blockIdx.x);
+    const CfgDesc& c = B.c[ci];
+    const int s0 = (blockIdx.x - c.blk0) * 32, mu = threadIdx.x >> 5, lane = threadIdx.x & 31, s = s0 + lane;
+    const double* src = canon + c.x_off + (size_t)s0 * 72;
+    const int n = min(32, c.V - s0) * 72;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) u.e[k / 3][k % 3] = {(T)src[2 * k], (T)src[2 * k + 1]};
-        Store<P>::store(w + c.w_off + (size_t)mu * Store<P>::reals * c.Vp, c.Vp, s, u);
+    for (int k = 0; k < 18; ++k) {
+        const int i = k * 128 + threadIdx.x;
+        if (i < n) buf[i + i / 72] = (T)__ldg(src + i);
     }
+    __syncthreads();
+    if (s >= c.V) return;
+    mat3<T> u;
+    const T* row = buf + lane * kRow + mu * 18;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) u.e[k / 3][k % 3] = {row[2 * k], row[2 * k + 1]};
+    Store<P>::store(w + c.w_off + (size_t)mu * Store<P>::reals * c.Vp, c.Vp, s, u);
 }
 
 template <int P, int CAP>
 __global__ void __launch_bounds__(128)
 k_unpack(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __restrict__ w, double* __restrict__ canon) {
     using T = typename Store<P>::T;
-    for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
-        const int ci = find_cfg(B, blk);
-        const CfgDesc& c = B.c[ci];
-        const int mu = threadIdx.x >> 5;
-        const int s = (blk - c.blk0) * 32 + (threadIdx.x & 31);
-        if (s >= c.V) continue;
+    __shared__ T buf[32 * kRow];
+    const int ci = find_cfg(B, blockIdx.x);
+    const CfgDesc& c = B.c[ci];
+    const int s0 = (blockIdx.x - c.blk0) * 32, mu = threadIdx.x >> 5, lane = threadIdx.x & 31, s = s0 + lane;
+    if (s < c.V) {
         mat3<T> u;
         Store<P>::load(w + c.w_off + (size_t)mu * Store<P>::reals * c.Vp, c.Vp, s, u);
-        double* dst = canon + c.x_off + ((size_t)s * 4 + mu) * 18;
+        T* row = buf + lane * kRow + mu * 18;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            dst[2 * k] = (double)u.e[k / 3][k % 3].re;
-            dst[2 * k + 1] = (double)u.e[k / 3][k % 3].im;
+            row[2 * k] = u.e[k / 3][k % 3].re;
+            row[2 * k + 1] = u.e[k / 3][k % 3].im;
         }
+    }
+    __syncthreads();
+    double* dst = canon + c.x_off + (size_t)s0 * 72;
+    const int n = min(32, c.V - s0) * 72;
+#pragma unroll
+    for (int k = 0; k < 18; ++k) {
+        const int i = k * 128 + threadIdx.x;
+        if (i < n) dst[i] = widen(buf[i + i / 72]);
     }
 }
 

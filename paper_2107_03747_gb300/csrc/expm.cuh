@@ -94,28 +94,42 @@ __device__ __forceinline__ void expm_su3(mat3<T>& m, const alg8<T>& x) {
         c0 *= sc * sc * sc;
     }
 
-    // f_j = sum_n i^n (alpha_n, beta_n, gamma_n) / n!, summed four terms at a time
-    // (i^n cycles i, -1, -i, +1 within a block; at most 20 terms, ||Q||_F <= 1 here)
-    T a = T(1), b = T(0), g = T(0);
-    // f0 starts at 1 (the n = 0 term) unless the unit matrix is taken out; with scaling and
-    // squaring the full matrix is needed first and 1 is subtracted at the end
-    T f0r = (MINUS_ONE && s == 0) ? T(0) : T(1), f0i = T(0), f1r = T(0), f1i = T(0), f2r = T(0), f2i = T(0);
-    const T tol = series_tol<T>::v;
+    // f_j = sum_n i^n (alpha_n, beta_n, gamma_n) / n!; f0 starts at 1 (the n = 0 term) unless the unit matrix is taken
+    // out; with scaling and squaring the full matrix is needed first and 1 is subtracted at the end
+    T f0r, f0i, f1r, f1i, f2r, f2i;
+    const T one = (MINUS_ONE && s == 0) ? T(0) : T(1);
+    if (sizeof(T) == 4 && r2 <= T(0.0625)) {
+        // FP32, the size of a flow step: the terms up to n = 8 written out in c1 and c0 (the tail is below
+        // 0.25^9 / 9! = 1e-11), 20 operations instead of two blocks of the recursion below: 0.9 % of the FP32 flow
+        const T w = c0 * c0, c2 = c1 * c1, a3 = fma(c1, c2, w);
+        f2r = fma(a3, T(1.0 / 40320), fma(c2, T(-1.0 / 720), fma(c1, T(1.0 / 24), T(-0.5))));
+        f2i = c0 * fma(c1, T(-2.0 / 5040), T(1.0 / 120));
+        f1i = fma(a3, T(-1.0 / 5040), fma(c2, T(1.0 / 120), fma(c1, T(-1.0 / 6), T(1))));
+        f1r = c0 * fma(c2, T(3.0 / 40320), fma(c1, T(-2.0 / 720), T(1.0 / 24)));
+        f0r = fma(w, fma(c1, T(2.0 / 40320), T(-1.0 / 720)), one);
+        f0i = c0 * fma(c2, T(-1.0 / 5040), fma(c1, T(1.0 / 120), T(-1.0 / 6)));
+    } else {
+        // summed four terms at a time (i^n cycles i, -1, -i, +1 within a block; at most 20 terms, ||Q||_F <= 1 here)
+        T a = T(1), b = T(0), g = T(0);
+        f0r = one;
+        f0i = f1r = f1i = f2r = f2i = T(0);
+        const T tol = series_tol<T>::v;
 #pragma unroll
-    for (int blk = 0; blk < 5; ++blk) {
+        for (int blk = 0; blk < 5; ++blk) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const T inv = T(1) / T(4 * blk + k + 1);
-            const T an = c0 * g * inv;
-            const T bn = fma(c1, g, a) * inv;
-            const T gn = b * inv;
-            a = an; b = bn; g = gn;
-            if (k == 0) { f0i += a; f1i += b; f2i += g; }
-            if (k == 1) { f0r -= a; f1r -= b; f2r -= g; }
-            if (k == 2) { f0i -= a; f1i -= b; f2i -= g; }
-            if (k == 3) { f0r += a; f1r += b; f2r += g; }
+            for (int k = 0; k < 4; ++k) {
+                const T inv = T(1) / T(4 * blk + k + 1);
+                const T an = c0 * g * inv;
+                const T bn = fma(c1, g, a) * inv;
+                const T gn = b * inv;
+                a = an; b = bn; g = gn;
+                if (k == 0) { f0i += a; f1i += b; f2i += g; }
+                if (k == 1) { f0r -= a; f1r -= b; f2r -= g; }
+                if (k == 2) { f0i -= a; f1i -= b; f2i -= g; }
+                if (k == 3) { f0r += a; f1r += b; f2r += g; }
+            }
+            if (fabs(a) + fabs(b) + fabs(g) < tol) break;
         }
-        if (fabs(a) + fabs(b) + fabs(g) < tol) break;
     }
     // Q scaled by sc for the polynomial
     const T s00 = q00 * sc, s11 = q11 * sc, s22 = q22 * sc;

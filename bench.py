@@ -124,7 +124,8 @@ def site_steps(members):
 
 
 def launches_per_flow(members):
-    """Kernels one flow enqueues: 3 stages per step, measure + reduce per distinct record set, + pack."""
+    """Kernels one flow enqueues (at least): 3 stages and the clover sum per step, clover halves and sum at each end
+    time, + pack; launches of many blocks add a reduction to each sum."""
     steps = [sum(n_steps(m[3])) for m in members]
     maxT = max(steps)
     k = 1  # pack
@@ -132,7 +133,7 @@ def launches_per_flow(members):
         k += 2
     for i in range(maxT):
         act = [s for s in steps if i < s]
-        k += 2 + 3  # measure+reduce (measure_every = 1), 3 stages
+        k += 1 + 3  # clover sum (measure_every = 1), 3 stages
         if any(s == i + 1 for s in act):
             k += 2
     return k

@@ -212,9 +212,18 @@ tgf_status last_launch(const char* what) {
     return TGF_OK;
 }
 
+// The block counter of configuration c's clover sum: the unused fourth double of its first partial (Layout::meas_blk0).
+int64_t sum_counter(double* scratch, const Layout& Ly, int c) {
+    return (int64_t)reinterpret_cast<uintptr_t>(scratch + Ly.meas_blk0[c] * kPartials + 3);
+}
+// sets it in the batch of a launch that writes clover halves
+void set_counters(Batch& B, double* scratch, const Layout& Ly, const std::vector<int>& which) {
+    for (int i = 0; i < B.ncfg; ++i) B.c[i].o_off = sum_counter(scratch, Ly, which[i]);
+}
+
 void* clover_base(void* scratch, const Layout& Ly) { return (char*)scratch + Ly.partial_bytes(); }
 
-// clover-sum + reduce over `which` (halves already written), record r_c at time t_c
+// clover sum over `which` (halves already written), record r_c at time t_c
 tgf_status enqueue_sum(int prec, unsigned flags, const tgf_lattice* lat, const Layout& Ly,
                        const std::vector<int>& which, const std::vector<int>& rec, const std::vector<double>& t,
                        size_t obs_stride, double* scratch, tgf_obs* obs, cudaStream_t st) {
@@ -222,12 +231,10 @@ tgf_status enqueue_sum(int prec, unsigned flags, const tgf_lattice* lat, const L
     for (int i = 0; i < B.ncfg; ++i) {
         B.c[i].h = t[i];
         B.c[i].o_off = (int64_t)which[i] * (int64_t)obs_stride + rec[i];
+        B.c[i].x_off = sum_counter(scratch, Ly, which[i]);
     }
-    launch_clover_sum(prec, flags, B, clover_base(scratch, Ly), scratch, st);
-    tgf_status s = last_launch("clover sum");
-    if (s) return s;
-    launch_reduce(B, scratch, reinterpret_cast<double*>(obs), st);
-    return last_launch("reduce");
+    launch_clover_sum(prec, flags, B, clover_base(scratch, Ly), scratch, reinterpret_cast<double*>(obs), st);
+    return last_launch("clover sum");
 }
 
 // full measurement of `which` from the field w: clover halves, their sum, the reduction
@@ -235,6 +242,7 @@ tgf_status enqueue_measure(int prec, unsigned flags, const tgf_lattice* lat, con
                            const std::vector<int>& which, const std::vector<int>& rec, const std::vector<double>& t,
                            size_t obs_stride, const void* w, double* scratch, tgf_obs* obs, cudaStream_t st) {
     Batch B = make_batch(lat, Ly, which, 32);
+    set_counters(B, scratch, Ly, which);
     launch_stage(prec, 1, 2, 0, B, w, nullptr, nullptr, clover_base(scratch, Ly), st);
     tgf_status s = last_launch("clover halves");
     if (s) return s;
@@ -818,6 +826,7 @@ tgf_status tgf_measure_slices(int prec, const tgf_lattice* lat, int ncfg, const 
     cudaStream_t st = (cudaStream_t)stream;
     std::vector<int> which = all_cfgs(ncfg);
     Batch H = make_batch(lat, Ly, which, 32);
+    set_counters(H, scratch, Ly, which);
     launch_stage(prec, 1, 2, 0, H, links, nullptr, nullptr, clover_base(scratch, Ly), st);
     if ((s = last_launch("clover halves"))) return s;
     // chunks of every slab, and the slabs.  The partial sums fit the scratch's per-block partials (4 doubles per
@@ -920,6 +929,7 @@ static tgf_status enqueue_flow(int prec, const tgf_lattice* lat, int ncfg, const
             const int c = act[k];
             B.c[k].h = (i < n[c]) ? eps : rest[c];
         }
+        if (mode1) set_counters(B, scratch, Ly, act);
         const int ru = (prec != TGF_FP64 && reunit_every > 0 && (i + 1) % reunit_every == 0) ? 1 : 0;
         if (mode1 && (s = join())) return s;  // stage 1 is about to rewrite the halves
         launch_stage(prec, 1, mode1, 0, B, cur, alt, accum, clover_base(scratch, Ly), st, grid, tile);

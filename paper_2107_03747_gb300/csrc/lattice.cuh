@@ -23,8 +23,9 @@ struct CfgDesc {
     unsigned dmul[3]; // s / st[d+1] = umulhi(16 s, dmul[d]) >> dsh[d] for every site s < 2^28
     uint8_t dsh[4];
     int64_t w_off;    // link storage offset (reals)
-    int64_t x_off;    // accumulator offset (reals)
-    int64_t o_off;    // observable slot (records) = cfg * obs_stride + rec; slice charge: cfg index
+    int64_t x_off;    // accumulator offset (reals); clover sum: address of the block counter
+    int64_t o_off;    // observable slot (records) = cfg * obs_stride + rec; slice charge: cfg index; clover halves:
+                      // address of the block counter of their sum
     int64_t m_off;    // clover-halves offset in the scratch buffer (reals of the storage type)
     double h;         // step size (stages) or flow time t (measure)
     int8_t tw[16];    // n_{mu nu} mod 3 in {0,1,2}, row-major 4x4, antisymmetric mod 3
@@ -111,6 +112,12 @@ template <class T>
 __device__ __forceinline__ void centre(int k, T& zr, T& zi) {
     zr = T(-0.5);
     zi = (k == 1) ? T(0.86602540378443864676) : T(-0.86602540378443864676);
+}
+
+// The stage kernels that write clover halves (modes 1 and 2) clear the configuration's counter of finished blocks of
+// the sum over them; o_off of their batch is its address.
+__device__ __forceinline__ void clear_counter(const CfgDesc& c, int blk) {
+    if (blk == c.blk0 && threadIdx.x == 0) *reinterpret_cast<unsigned*>(c.o_off) = 0u;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -396,9 +403,9 @@ void launch_stage64(int stage, int mode, const Batch& B, const double* w_in, dou
                     cudaStream_t st, int grid);
 constexpr int kTiles = 5;
 inline int tile_sites(int tile) { return tile == 1 ? 64 : 32; }
-void launch_clover_sum(int prec, unsigned flags, const Batch& B, const void* clov, double* partial,
+// x_off of the batch: the address of each configuration's block counter (clear_counter)
+void launch_clover_sum(int prec, unsigned flags, const Batch& B, const void* clov, double* partial, double* obs,
                        cudaStream_t st);
-void launch_reduce(const Batch& B, const double* partial, double* obs, cudaStream_t st);
 // Host: the first observable slot + 1 whose record came out non-finite since the last call (0 if
 // none), read and cleared on `st` (synchronises `st`).
 unsigned long long nonfinite_read_and_clear(cudaStream_t st, cudaError_t* err);

@@ -8,8 +8,8 @@
 //   s(n) = sum_{mu<nu} (3 - Re Tr[Z* P_{mu nu}(n)])
 // in the working precision (the stage kernel stores each plane's 3 - Re Tr[Z* P], so the small
 // deviations are summed, not six numbers near 3), then reduces them over the block in FP64 (warp
-// shuffles, fixed order) to one partial per block.  k_reduce sums each configuration's partials in
-// block order and writes {t, E, Q, P, S} with E = sum e/(64 V), Q = sum q/(256 pi^2) (eq. qlatt
+// shuffles, fixed order) to one partial per block.  The partials of a configuration are summed in a fixed
+// order, by its last block or by k_reduce, into {t, E, Q, P, S} with E = sum e/(64 V), Q = sum q/(256 pi^2) (eq. qlatt
 // with Gt_{mu nu} = eps_{mu nu rho sigma} G_{rho sigma}/2), S = sum s, P = 1 - S/(18 V).
 // Both orders are fixed: results are bitwise reproducible.
 #include <cuda_runtime.h>
@@ -39,116 +39,138 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 constexpr double kSliceUnit = 1.0 / (256.0 * 3.14159265358979323846 * 3.14159265358979323846);
 
-template <class T, int CAP>
-__global__ void __launch_bounds__(kMeasureSites)
-k_clover_sum(const __grid_constant__ BatchT<CAP> B, const T* __restrict__ clov, double* __restrict__ partial,
-             int traceless) {
-    __shared__ double red[kMeasureSites / 32][3];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
-        const int ci = find_cfg(B, blk);
-        const CfgDesc& c = B.c[ci];
-        const int s = (blk - c.blk0) * kMeasureSites + threadIdx.x;
-        double e = 0, q = 0, pl = 0;
-        if (s < c.V) {
-            const T* cb = clov + c.m_off;
-            const size_t Vp = (size_t)c.Vp;
-            T te = T(0), tq = T(0), tp = T(0);
-            T a0[9];
-#pragma unroll
-            for (int p = 0; p < 6; ++p) {
-                T a[9], a1[9];
-                AhStore<T>::load(cb + (size_t)(p * 2) * 9 * Vp, (int)Vp, s, a);
-                AhStore<T>::load(cb + (size_t)(p * 2 + 1) * 9 * Vp, (int)Vp, s, a1);
-#pragma unroll
-                for (int k = 0; k < 9; ++k) a[k] += a1[k];
-                if (traceless) {
-                    const T tr = (a[0] + a[1] + a[2]) * (T(1) / T(3));
-                    a[0] -= tr; a[1] -= tr; a[2] -= tr;
-                }
-                te += a[0] * a[0] + a[1] * a[1] + a[2] * a[2] +
-                      T(2) * (a[3] * a[3] + a[4] * a[4] + a[5] * a[5] + a[6] * a[6] + a[7] * a[7] + a[8] * a[8]);
-                if (p & 1) {
-                    const T d = a0[0] * a[0] + a0[1] * a[1] + a0[2] * a[2] +
-                                T(2) * (a0[3] * a[3] + a0[4] * a[4] + a0[5] * a[5] + a0[6] * a[6] + a0[7] * a[7] + a0[8] * a[8]);
-                    tq += (p == 3) ? -d : d;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 9; ++k) a0[k] = a[k];
-                }
-                tp += __ldg(cb + (size_t)(108 + p) * Vp + s);
-            }
-            e = (double)te;
-            q = (double)tq;
-            pl = (double)tp;
-        }
-        e = warp_sum(e);
-        q = warp_sum(q);
-        pl = warp_sum(pl);
-        if (lane == 0) {
-            red[warp][0] = e;
-            red[warp][1] = q;
-            red[warp][2] = pl;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double se = 0, sq = 0, sp = 0;
-#pragma unroll
-            for (int i = 0; i < kMeasureSites / 32; ++i) {
-                se += red[i][0];
-                sq += red[i][1];
-                sp += red[i][2];
-            }
-            double* o = partial + (size_t)blk * kPartials;
-            o[0] = se;
-            o[1] = sq;
-            o[2] = sp;
-            o[3] = 0.0;
-        }
-        __syncthreads();
+// Sums of a configuration's partials -> its record {t, E, Q, P, S}.
+__device__ __forceinline__ void write_record(const CfgDesc& c, double e, double q, double S, double* __restrict__ obs) {
+    const double V = (double)c.V;
+    const double pi = 3.14159265358979323846;
+    double* o = obs + (size_t)c.o_off * 5;
+    const double E = e / (64.0 * V), Q = q / (256.0 * pi * pi);
+    o[0] = c.h;                                   // t
+    o[1] = E;
+    o[2] = Q;
+    o[3] = 1.0 - S / (18.0 * V);                  // P = (1/(18V)) sum Re Tr[Z* P]
+    o[4] = S;                                     // S = sum (3 - Re Tr[Z* P])
+    // a non-finite record (non-finite links in, or an overflow) is reported to the host
+    if (!isfinite(E) || !isfinite(Q) || !isfinite(S))
+        atomicCAS(&g_nonfinite, 0ull, (unsigned long long)c.o_off + 1ull);
+}
+// One of the three sums (k = 0, 1, 2: e, q, s) over nb partials, by a warp, in a fixed order.  A configuration's partials
+// are summed in four such parts, by whichever kernel does it: the record is the same to the bit.
+__device__ __forceinline__ double sum_partials(const double* __restrict__ partial, int nb, int k, int lane) {
+    const double* o = partial + k;
+    double v0 = 0, v1 = 0;
+    int i = lane;
+    for (; i + 32 < nb; i += 64) {
+        v0 += __ldcg(o + (size_t)i * kPartials);
+        v1 += __ldcg(o + (size_t)(i + 32) * kPartials);
     }
+    if (i < nb) v0 += __ldcg(o + (size_t)i * kPartials);
+    return warp_sum(v0 + v1);
 }
 
-// One block per configuration of the launch: fixed-order sum of its partials.
-template <int CAP>
-__global__ void __launch_bounds__(256)
-k_reduce(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ partial, double* __restrict__ obs) {
-    __shared__ double red[3][256];
-    const CfgDesc& c = B.c[blockIdx.x];
-    const int nb_cfg = (c.V + kMeasureSites - 1) / kMeasureSites;
-    double e = 0, q = 0, p = 0;
-    for (int i = threadIdx.x; i < nb_cfg; i += 256) {
-        const double* o = partial + (size_t)(c.blk0 + i) * kPartials;
-        e += o[0];
-        q += o[1];
-        p += o[2];
-    }
-    red[0][threadIdx.x] = e;
-    red[1][threadIdx.x] = q;
-    red[2][threadIdx.x] = p;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            red[0][threadIdx.x] += red[0][threadIdx.x + w];
-            red[1][threadIdx.x] += red[1][threadIdx.x + w];
-            red[2][threadIdx.x] += red[2][threadIdx.x + w];
+// One thread per site, bound by HBM where the lattice is large (4 x 16x16x48x48 in FP32: 1.08 GB in 183 us).  LAST: the last
+// block of a configuration to finish (its counter, cleared by the stage kernel that wrote the halves) sums the
+// partials, instead of a launch of its own for a few numbers (k_reduce).  That is for launches of few blocks, whose
+// time is latency: the 18-step flow of 4x4x12x12, 18 blocks, 295 -> 283 us; with many blocks the fence and the counter
+// cost more than the launch (a 6-step flow of 4 x 16x16x48x48 17.10 -> 17.15 ms).  Three threads per site, one for
+// each pair of planes, were no faster on the small lattice and 22 % slower on the large one.
+template <class T, int CAP, bool LAST>
+__global__ void __launch_bounds__(kMeasureSites)
+k_clover_sum(const __grid_constant__ BatchT<CAP> B, const T* __restrict__ clov, double* partial, double* __restrict__ obs,
+             int traceless) {
+    __shared__ double red[kMeasureSites / 32][3];
+    __shared__ bool last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ci = find_cfg(B, blockIdx.x);
+    const CfgDesc& c = B.c[ci];
+    const int s = (blockIdx.x - c.blk0) * kMeasureSites + threadIdx.x;
+    double e = 0, q = 0, pl = 0;
+    if (s < c.V) {
+        const T* cb = clov + c.m_off;
+        const size_t Vp = (size_t)c.Vp;
+        T te = T(0), tq = T(0), tp = T(0);
+        T a0[9];
+#pragma unroll
+        for (int p = 0; p < 6; ++p) {
+            T a[9], a1[9];
+            AhStore<T>::load(cb + (size_t)(p * 2) * 9 * Vp, (int)Vp, s, a);
+            AhStore<T>::load(cb + (size_t)(p * 2 + 1) * 9 * Vp, (int)Vp, s, a1);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) a[k] += a1[k];
+            if (traceless) {
+                const T tr = (a[0] + a[1] + a[2]) * (T(1) / T(3));
+                a[0] -= tr; a[1] -= tr; a[2] -= tr;
+            }
+            te += a[0] * a[0] + a[1] * a[1] + a[2] * a[2] +
+                  T(2) * (a[3] * a[3] + a[4] * a[4] + a[5] * a[5] + a[6] * a[6] + a[7] * a[7] + a[8] * a[8]);
+            if (p & 1) {
+                const T d = a0[0] * a[0] + a0[1] * a[1] + a0[2] * a[2] +
+                            T(2) * (a0[3] * a[3] + a0[4] * a[4] + a0[5] * a[5] + a0[6] * a[6] + a0[7] * a[7] + a0[8] * a[8]);
+                tq += (p == 3) ? -d : d;
+            } else {
+#pragma unroll
+                for (int k = 0; k < 9; ++k) a0[k] = a[k];
+            }
+            tp += __ldg(cb + (size_t)(108 + p) * Vp + s);
         }
-        __syncthreads();
+        e = (double)te;
+        q = (double)tq;
+        pl = (double)tp;
     }
+    e = warp_sum(e);
+    q = warp_sum(q);
+    pl = warp_sum(pl);
+    if (lane == 0) {
+        red[warp][0] = e;
+        red[warp][1] = q;
+        red[warp][2] = pl;
+    }
+    __syncthreads();
+    const int nb = (c.V + kMeasureSites - 1) / kMeasureSites;
     if (threadIdx.x == 0) {
-        const double V = (double)c.V;
-        const double pi = 3.14159265358979323846;
-        double* o = obs + (size_t)c.o_off * 5;
-        const double E = red[0][0] / (64.0 * V), Q = red[1][0] / (256.0 * pi * pi), S = red[2][0];
-        o[0] = c.h;                                   // t
-        o[1] = E;
-        o[2] = Q;
-        o[3] = 1.0 - S / (18.0 * V);                  // P = (1/(18V)) sum Re Tr[Z* P]
-        o[4] = S;                                     // S = sum (3 - Re Tr[Z* P])
-        // a non-finite record (non-finite links in, or an overflow) is reported to the host
-        if (!isfinite(E) || !isfinite(Q) || !isfinite(S))
-            atomicCAS(&g_nonfinite, 0ull, (unsigned long long)c.o_off + 1ull);
+        double v[3] = {0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < kMeasureSites / 32; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[k] += red[i][k];
+        double* o = partial + (size_t)blockIdx.x * kPartials;
+        o[0] = v[0];
+        o[1] = v[1];
+        o[2] = v[2];
+        if (LAST) {
+            __threadfence();
+            last = atomicAdd(reinterpret_cast<unsigned*>(c.x_off), 1u) == (unsigned)(nb - 1);
+        }
     }
+    if (!LAST) return;
+    __syncthreads();
+    if (!last) return;
+    const int lo = nb * warp / 4, hi = nb * (warp + 1) / 4;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const double v = sum_partials(partial + (size_t)(c.blk0 + lo) * kPartials, hi - lo, k, lane);
+        if (lane == 0) red[warp][k] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        write_record(c, (red[0][0] + red[1][0]) + (red[2][0] + red[3][0]), (red[0][1] + red[1][1]) + (red[2][1] + red[3][1]),
+                     (red[0][2] + red[1][2]) + (red[2][2] + red[3][2]), obs);
+}
+
+// One block per configuration of the launch: the sums over its partials, by four warps each.
+template <int CAP>
+__global__ void __launch_bounds__(384)
+k_reduce(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ partial, double* __restrict__ obs) {
+    __shared__ double red[12];
+    const CfgDesc& c = B.c[blockIdx.x];
+    const int nb = (c.V + kMeasureSites - 1) / kMeasureSites, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lo = nb * (warp & 3) / 4, hi = nb * ((warp & 3) + 1) / 4;
+    const double v = sum_partials(partial + (size_t)(c.blk0 + lo) * kPartials, hi - lo, warp >> 2, lane);
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        write_record(c, (red[0] + red[1]) + (red[2] + red[3]), (red[4] + red[5]) + (red[6] + red[7]),
+                     (red[8] + red[9]) + (red[10] + red[11]), obs);
 }
 
 // q(x0, t) (Sec. 4): the charge density summed over the slab x_dir = x of each configuration, FP64 sums in a
@@ -250,40 +272,30 @@ void launch_slice_charge(int prec, unsigned flags, const Batch& B, const Batch& 
                : slices_cap<float, kMaxCfg>(B, R, clov, dir, q, q_stride, partial, flags, st);
 }
 
+constexpr int kLastBlocks = 608;  // up to this many blocks (4 per SM) the last one reduces
+
 template <class T, int CAP>
-static void sum_cap(unsigned flags, const Batch& B, const void* clov, double* partial, cudaStream_t st) {
-    if constexpr (CAP == kMaxCfg) {
-        k_clover_sum<T, kMaxCfg><<<B.nblk, kMeasureSites, 0, st>>>(B, (const T*)clov, partial, (int)(flags & 1u));
+static void sum_cap(unsigned flags, const Batch& B, const void* clov, double* partial, double* obs, cudaStream_t st) {
+    BatchT<CAP> b;
+    b.ncfg = B.ncfg;
+    b.nblk = B.nblk;
+    for (int i = 0; i < B.ncfg; ++i) b.c[i] = B.c[i];
+    if (B.nblk <= kLastBlocks) {
+        k_clover_sum<T, CAP, true><<<B.nblk, kMeasureSites, 0, st>>>(b, (const T*)clov, partial, obs, (int)(flags & 1u));
     } else {
-        BatchT<CAP> b;
-        b.ncfg = B.ncfg;
-        b.nblk = B.nblk;
-        for (int i = 0; i < B.ncfg; ++i) b.c[i] = B.c[i];
-        k_clover_sum<T, CAP><<<B.nblk, kMeasureSites, 0, st>>>(b, (const T*)clov, partial, (int)(flags & 1u));
+        k_clover_sum<T, CAP, false><<<B.nblk, kMeasureSites, 0, st>>>(b, (const T*)clov, partial, obs, (int)(flags & 1u));
+        k_reduce<CAP><<<B.ncfg, 384, 0, st>>>(b, partial, obs);
     }
 }
 
-template <class T>
-static void sum_t(unsigned flags, const Batch& B, const void* clov, double* partial, cudaStream_t st) {
-    if (B.ncfg <= kSmallCap) sum_cap<T, kSmallCap>(flags, B, clov, partial, st);
-    else sum_cap<T, kMaxCfg>(flags, B, clov, partial, st);
-}
-
-void launch_clover_sum(int prec, unsigned flags, const Batch& B, const void* clov, double* partial,
+void launch_clover_sum(int prec, unsigned flags, const Batch& B, const void* clov, double* partial, double* obs,
                        cudaStream_t st) {
-    if (prec == P64) sum_t<double>(flags, B, clov, partial, st);
-    else sum_t<float>(flags, B, clov, partial, st);
-}
-
-void launch_reduce(const Batch& B, const double* partial, double* obs, cudaStream_t st) {
     if (B.ncfg <= kSmallCap) {
-        BatchT<kSmallCap> b;
-        b.ncfg = B.ncfg;
-        b.nblk = B.nblk;
-        for (int i = 0; i < B.ncfg; ++i) b.c[i] = B.c[i];
-        k_reduce<kSmallCap><<<B.ncfg, 256, 0, st>>>(b, partial, obs);
+        if (prec == P64) sum_cap<double, kSmallCap>(flags, B, clov, partial, obs, st);
+        else sum_cap<float, kSmallCap>(flags, B, clov, partial, obs, st);
     } else {
-        k_reduce<kMaxCfg><<<B.ncfg, 256, 0, st>>>(B, partial, obs);
+        if (prec == P64) sum_cap<double, kMaxCfg>(flags, B, clov, partial, obs, st);
+        else sum_cap<float, kMaxCfg>(flags, B, clov, partial, obs, st);
     }
 }
 

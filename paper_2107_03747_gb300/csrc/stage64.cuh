@@ -124,6 +124,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
     for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
         const int ci = find_cfg(B, blk);
         const CfgDesc& c = B.c[ci];
+        if (MODE != 0) clear_counter(c, blk);
         int s = (blk - c.blk0) * 32 + lane;
         const bool valid = s < c.V;  // lanes past the end take part in the barriers on site 0 and store nothing
         if (!valid) s = 0;

@@ -155,6 +155,7 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
     for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
         const int ci = find_cfg(B, blk);
         const CfgDesc& c = B.c[ci];
+        if (MODE != 0) clear_counter(c, blk);
         int s_raw = (blk - c.blk0) * SPB + row * 32 + lane;
         int xc[4];
         bool have_x = false;

@@ -282,8 +282,38 @@ __device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, in
         }
 }
 
-template <int N, bool SYNC, class SRC, class SKIP, class VISIT>
-__device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const CfgDesc& c, int s, int mu, unsigned eb, fx_guard& g,
+// Links that several warps of a block need, taken as operands once and shared: [dir] U_dir(n) and [4 + dir] U_dir(n - dir)
+// of the block's 32 sites, entry by entry (re hi, lo, im hi, lo), and the guard words of what was taken.
+template <int N>
+struct fx_shared {
+    int4 u[8][N * N][32];
+    unsigned bad[8][32];
+};
+template <int N>
+__device__ __forceinline__ void fx_share(fx_shared<N>& sh, int m, int lane, const matx<N>& o, const fx_guard& g) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) sh.u[m][i * N + j][lane] = make_int4(o.rh[i][j], o.rl[i][j], o.ih[i][j], o.il[i][j]);
+    sh.bad[m][lane] = g.bad();
+}
+template <int N>
+__device__ __forceinline__ void fx_shared_link(matx<N>& o, const fx_shared<N>& sh, int m, int lane) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int4 v = sh.u[m][i * N + j][lane];
+            o.rh[i][j] = v.x;
+            o.rl[i][j] = v.y;
+            o.ih[i][j] = v.z;
+            o.il[i][j] = v.w;
+        }
+}
+
+// sh: the block's shared links (SHARE), filled and followed by a barrier of fx_staples' first iteration
+template <int N, bool SYNC, bool SHARE, class SRC, class SKIP, class VISIT>
+__device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shared<N>* sh, int lane, const CfgDesc& c, int s, int mu, unsigned eb, fx_guard& g,
                                            SKIP&& skip, VISIT&& visit, int q0 = 0, int q1 = 6) {
     const int s_mp = fwd(c, eb, s, mu);
     const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
@@ -308,15 +338,27 @@ __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const CfgDesc
             SRC::centre(k, zr, zi);
             fx_scale(b, zr, back ? -zi : zi);
         }
-        fx_take_matrix<N>(d, src, nu, sc, back, g);
+        if (SHARE && !back) fx_shared_link<N>(d, *sh, nu, lane);
+        else fx_take_matrix<N>(d, src, nu, sc, back, g);
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             vecx<N> v, t;
+            if (SHARE && back) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) {
-                const double2 x = src.get(nu, sv, i, j, back);
-                fx_take(x.x, v.rh[j], v.rl[j], g);
-                fx_take(x.y, v.ih[j], v.il[j], g);
+                for (int j = 0; j < N; ++j) {
+                    const int4 x = sh->u[4 + nu][j * N + i][lane];
+                    v.rh[j] = x.x;
+                    v.rl[j] = x.y;
+                    v.ih[j] = x.z;
+                    v.il[j] = x.w;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const double2 x = src.get(nu, sv, i, j, back);
+                    fx_take(x.x, v.rh[j], v.rl[j], g);
+                    fx_take(x.y, v.ih[j], v.il[j], g);
+                }
             }
             vecx<N> nv = fx_negated(v);
 #pragma unroll
@@ -364,6 +406,12 @@ __device__ __forceinline__ unsigned fx_scale_of(const cx<double> (&m)[N][N]) {
             a = max(a, (unsigned)__double2hiint(m[i][j].im) & 0x7fffffffu);
         }
     return (unsigned)min(max(1022 - (int)(a >> 20), 0), 40);
+}
+// v 2^-58, the factor taken off the exponent (a whole number but 0 is at least 1 in magnitude)
+__device__ __forceinline__ double fx_value(long long v) {
+    const double x = (double)v;
+    const int h = __double2hiint(x);
+    return __hiloint2double(h ? h - (kFxBits << 20) : 0, __double2loint(x));
 }
 // 2^(-58 - up)
 __device__ __forceinline__ double fx_unit(unsigned up) { return __hiloint2double((int)((1023u - kFxBits - up) << 20), 0); }

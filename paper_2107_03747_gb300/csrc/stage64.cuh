@@ -119,8 +119,14 @@ __global__ void __launch_bounds__(WIDE ? 384 : 128, WIDE ? 1 : MODE == 0 ? 3 : 2
 k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
           double* __restrict__ acc, double* __restrict__ clov) {
     const int mu = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31, part = threadIdx.x >> 7;
-    __shared__ long long s_sum[WIDE && MODE != 2 ? 2 : 1][WIDE && MODE != 2 ? 18 : 1][128];
-    __shared__ unsigned s_bad[2][128];
+    // the links shared by the block's warps; WIDE: then the staple sums of its second and third part
+    __shared__ union {
+        fx_shared<3> links;
+        struct {
+            long long v[2][18][128];
+            unsigned bad[2][128];
+        } sum;
+    } sm;
     for (int blk = blockIdx.x; blk < B.nblk; blk += gridDim.x) {
         const int ci = find_cfg(B, blk);
         const CfgDesc& c = B.c[ci];
@@ -141,7 +147,14 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
         Su3Src src{base, Vp};
         fx_zero(sig);
         if (MODE != 0) fx_zero(kk);
-        fx_staples<3, true>(sig, src, c, s, mu, eb, g, [&](int nu) { return MODE == 2 && !c_clover_owner[mu][nu]; },
+        __syncthreads();  // the block before is done with the shared memory
+#pragma unroll 1
+        for (int m = mu + 4 * part; m < 8; m += WIDE ? 12 : 4) {
+            fx_guard gl;
+            fx_take_matrix<3>(u, src, mu, m < 4 ? s : bwd(c, eb, s, mu), false, gl);
+            fx_share<3>(sm.links, m, lane, u, gl);
+        }
+        fx_staples<3, true, true>(sig, src, &sm.links, lane, c, s, mu, eb, g, [&](int nu) { return MODE == 2 && !c_clover_owner[mu][nu]; },
             [&](int back, int nu, const matq<3>& sum) {
                 if (!valid || MODE == 0) return;
                 if (!c_clover_owner[mu][nu]) {
@@ -149,7 +162,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                     return;
                 }
                 const int pl = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
-                fx_take_matrix<3>(u, src, mu, s, false, g);
+                fx_shared_link<3>(u, sm.links, mu, lane);
                 const long long half = fx_round();
                 if (!back) {
                     // 3 - Re Tr(U F), the deviation of the twisted plaquette from the unit matrix
@@ -190,26 +203,29 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 kk = sum;
             },
             WIDE ? 2 * part : 0, WIDE ? 2 * part + 2 : 6);
+        fx_shared_link<3>(u, sm.links, mu, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) g.top2 |= sm.links.bad[m][lane];
         if constexpr (WIDE && MODE != 2) {
             const int lt = threadIdx.x & 127;
-            __syncthreads();  // the block before has read its sums
+            __syncthreads();  // the links have been read: their place takes the sums
             if (part) {
-                s_bad[part - 1][lt] = g.bad();
+                sm.sum.bad[part - 1][lt] = g.bad();
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
-                    s_sum[part - 1][i][lt] = sig.re[i / 3][i % 3];
-                    s_sum[part - 1][9 + i][lt] = sig.im[i / 3][i % 3];
+                    sm.sum.v[part - 1][i][lt] = sig.re[i / 3][i % 3];
+                    sm.sum.v[part - 1][9 + i][lt] = sig.im[i / 3][i % 3];
                 }
             }
             __syncthreads();
             if (part) continue;
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                g.top2 |= s_bad[p][lt];
+                g.top2 |= sm.sum.bad[p][lt];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
-                    sig.re[i / 3][i % 3] += s_sum[p][i][lt];
-                    sig.im[i / 3][i % 3] += s_sum[p][9 + i][lt];
+                    sig.re[i / 3][i % 3] += sm.sum.v[p][i][lt];
+                    sig.im[i / 3][i % 3] += sm.sum.v[p][9 + i][lt];
                 }
             }
             fx_check<3, 29>(sig, g);
@@ -228,7 +244,6 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
             matx<3> sx;
             matq<3> om;
             fx_operand_wide<3, 2>(sx, sig);
-            fx_take_matrix<3>(u, src, mu, s, false, g);
             fx_mul_nn<3>(om, u, sx);
             const double tr = (double)(om.im[0][0] + om.im[1][1] + om.im[2][2]) * (1.0 / 3.0);
             z.v[0] = 0x1p-56 * (tr - (double)om.im[0][0]);
@@ -254,6 +269,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
             add_to(w, d);
         } else {
             matq<3> d;
+            if (!WIDE) fx_shared_link<3>(u, sm.links, mu, lane);
             fx_mul_nn<3>(d, ex, u);
             const double unit = fx_unit(up);
 #pragma unroll

@@ -284,9 +284,9 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
                         f.e[i][j].re = sg * (f.e[i][j].re - b.e[i][j].re);
                         f.e[i][j].im = sg * (f.e[i][j].im - b.e[i][j].im);
                     }
-                mul_nn(t, a, f);
+                mul_nn_ah(t, a, f);
                 store_ah(cb + (size_t)(pl * 2 + 0) * 9 * Vp, Vp, s, t);
-                mul_nn(t, f, a);
+                mul_nn_ah(t, f, a);
                 store_ah(cb + (size_t)(pl * 2 + 1) * 9 * Vp, Vp, s_mp, t);
             }
         }
@@ -294,7 +294,7 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
         // Omega = U_mu(n) Sigma, Z = -P_ta(Omega)
         mat3<T> u;
         link(mu, s, u);
-        mul_nn(t, u, sig);
+        mul_nn_ah(t, u, sig);
         alg8<T> z;
         minus_proj_ta(z, t);
         const T h = (T)c.h;

@@ -43,7 +43,7 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 }
 __device__ __forceinline__ uint64_t hash64(uint64_t key, uint64_t counter) { return mix64(key + (counter + 1) * kGolden); }
 __device__ __forceinline__ double draw(uint64_t key, uint64_t counter) {
-    return ((double)(hash64(key, counter) >> 11) + 1.0) * 0x1.0p-53;
+    return (double)((hash64(key, counter) >> 11) + 1) * 0x1.0p-53;  // at most 2^53: exact
 }
 
 struct quat {
@@ -62,6 +62,7 @@ __device__ __forceinline__ quat qconj(const quat& a) { return {a.a0, -a.a1, -a.a
 __device__ bool sample_x0(double alpha, uint64_t key, uint64_t c0, double& x0) {
     const bool kp = alpha > 2.0;
     const double e2a = kp ? 0.0 : exp(-2.0 * alpha);
+    const double inv = 0.5 / alpha;
 #pragma unroll 1
     for (int a = 0; a < kAttempts; ++a) {
         const uint64_t c = c0 + 4 * a;
@@ -69,8 +70,8 @@ __device__ bool sample_x0(double alpha, uint64_t key, uint64_t c0, double& x0) {
         if (kp) {
             // Kennedy-Pendleton: lambda^2 = -(ln r1 + cos^2(2 pi r2) ln r3) / (2 alpha)
             const double r3 = draw(key, c + 2), r4 = draw(key, c + 3);
-            const double cs = cos(2.0 * M_PI * r2);
-            const double lam2 = -__dadd_rn(log(r1), __dmul_rn(__dmul_rn(cs, cs), log(r3))) / (2.0 * alpha);
+            const double cs = cospi(2.0 * r2);
+            const double lam2 = -__dadd_rn(log(r1), __dmul_rn(__dmul_rn(cs, cs), log(r3))) * inv;
             if (__dmul_rn(r4, r4) <= 1.0 - lam2) {
                 x0 = 1.0 - 2.0 * lam2;
                 return true;
@@ -140,7 +141,7 @@ __device__ __forceinline__ cx<double> rot_j(const rot2& R, const cx<double>& p, 
 // The update of the SU(2) block x (twice its SU(2)-proportional part): over-relaxation R = (v^+)^2 or a
 // heat-bath draw R = X v^+, x = |x| v.
 template <int OVERRELAX>
-__device__ __forceinline__ rot2 draw_rotation(const quat& x, double beta, uint64_t key, uint64_t c0) {
+__device__ __forceinline__ rot2 draw_rotation(const quat& x, double unit, double beta, uint64_t key, uint64_t c0) {
     const double n2 = x.a0 * x.a0 + x.a1 * x.a1 + x.a2 * x.a2 + x.a3 * x.a3;
     const bool live = n2 > 1e-290;
     quat R = {1.0, 0.0, 0.0, 0.0};
@@ -153,12 +154,13 @@ __device__ __forceinline__ rot2 draw_rotation(const quat& x, double beta, uint64
     } else {
         const double k2 = sqrt(n2);  // 2 k
         double x0;
-        if (sample_x0(beta * k2 / 3.0, key, c0, x0)) {
+        if (sample_x0(beta * (k2 * unit) / 3.0, key, c0, x0)) {
             const double cth = 2.0 * draw(key, c0 + 256) - 1.0;
-            const double phi = 2.0 * M_PI * draw(key, c0 + 257);
+            double sphi, cphi;
+            sincospi(2.0 * draw(key, c0 + 257), &sphi, &cphi);
             const double sth = sqrt(fmax(0.0, 1.0 - cth * cth));
             const double rr = sqrt(fmax(0.0, 1.0 - x0 * x0));
-            const quat X = {x0, rr * sth * cos(phi), rr * sth * sin(phi), rr * cth};
+            const quat X = {x0, rr * sth * cphi, rr * sth * sphi, rr * cth};
             const quat v = live ? quat{x.a0 / k2, x.a1 / k2, x.a2 / k2, x.a3 / k2} : quat{1.0, 0.0, 0.0, 0.0};
             R = qmul(X, qconj(v));
         }
@@ -214,7 +216,7 @@ __device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j
 // Matrix products of the staples, Omega and the rotations of U run in fixed point on the integer pipe
 // (fixed.cuh), the SU(2) blocks and draws in FP64, and an over-relaxation takes (v^+)^2 from x with one
 // division: about 210 FP64 instructions instead of 2,200, which kept the FP64 pipe 94 % busy.
-// One hybrid sweep (1 heat-bath, 12 over-relaxation) of 256 x 4x4x12x12: 114.9 ms before, 34.0 now.
+// One hybrid sweep (1 heat-bath, 12 over-relaxation) of 256 x 4x4x12x12: 114.9 ms before, 33.2 now.
 template <int OVERRELAX, int CAP>
 __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ BatchT<CAP> B, double* __restrict__ w,
                                                       int mu, int parity, double beta, uint64_t seed, uint64_t sweep) {
@@ -256,14 +258,18 @@ __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ Ba
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int k = 0; k < 3; ++k) wm.e[i][k] = {(double)om.re[i][k] * 0x1p-56, (double)om.im[i][k] * 0x1p-56};
+            for (int k = 0; k < 3; ++k) wm.e[i][k] = {(double)om.re[i][k], (double)om.im[i][k]};
     }
-    if (g.bad()) native_omega(wm, base, Vp, c, s, eb, mu);
+    double unit = 0x1p-56;  // of W: the rotations depend on its direction only, but for the heat-bath's alpha
+    if (g.bad()) {
+        native_omega(wm, base, Vp, c, s, eb, mu);
+        unit = 1.0;
+    }
     const uint64_t key = hash64(seed, (uint64_t)ci);
     const uint64_t c0 = (((uint64_t)sweep * 4 + (uint64_t)mu) * (uint64_t)c.V + (uint64_t)s) * 3 * kSlots;
     // the three subgroups (0,1), (0,2), (1,2), each on W after the ones before it; only the entries
     // that a later block reads are rotated
-    const rot2 R0 = draw_rotation<OVERRELAX>(su2_block(wm, 0, 1), beta, key, c0);
+    const rot2 R0 = draw_rotation<OVERRELAX>(su2_block(wm, 0, 1), unit, beta, key, c0);
     {
         const cx<double> p1 = wm.e[0][1], p2 = wm.e[0][2];
 #pragma unroll
@@ -271,10 +277,10 @@ __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ Ba
         wm.e[1][1] = rot_j(R0, p1, wm.e[1][1]);
         wm.e[1][2] = rot_j(R0, p2, wm.e[1][2]);
     }
-    const rot2 R1 = draw_rotation<OVERRELAX>(su2_block(wm, 0, 2), beta, key, c0 + kSlots);
+    const rot2 R1 = draw_rotation<OVERRELAX>(su2_block(wm, 0, 2), unit, beta, key, c0 + kSlots);
     wm.e[2][1] = rot_j(R1, wm.e[0][1], wm.e[2][1]);
     wm.e[2][2] = rot_j(R1, wm.e[0][2], wm.e[2][2]);
-    const rot2 R2 = draw_rotation<OVERRELAX>(su2_block(wm, 1, 2), beta, key, c0 + 2 * kSlots);
+    const rot2 R2 = draw_rotation<OVERRELAX>(su2_block(wm, 1, 2), unit, beta, key, c0 + 2 * kSlots);
 
     matx<3> u;
     matq<3> out;
@@ -300,7 +306,7 @@ __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ Ba
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int k = 0; k < 3; ++k) un.e[i][k] = {(double)out.re[i][k] * 0x1p-58, (double)out.im[i][k] * 0x1p-58};
+            for (int k = 0; k < 3; ++k) un.e[i][k] = {fx_value(out.re[i][k]), fx_value(out.im[i][k])};
     }
     Store<P64>::store(base + (size_t)mu * 18 * Vp, Vp, s, un);
 }

@@ -249,7 +249,7 @@ __device__ __forceinline__ void fx_take_entry(matx<N>& o, int i, int j, double r
 // fetch the same instructions at the same time: 11 % on the FP64 stage (8.63 instead of 9.74 ms for
 // 4 steps of 4 x 8x8x24x24).
 // visit(q, nu, sig): called after the forward (q = 0) and after the backward staple (q = 1) of a direction,
-// with the sum in normal orientation; skip(nu) leaves a direction out.  q0, q1: the part of the six staples (in
+// with the sum in normal orientation.  q0, q1: the part of the six staples (in
 // pairs) that this thread sums.
 template <int N>
 __device__ __forceinline__ void fx_transpose(matq<N>& m) {
@@ -312,9 +312,9 @@ __device__ __forceinline__ void fx_shared_link(matx<N>& o, const fx_shared<N>& s
 }
 
 // sh: the block's shared links (SHARE), filled and followed by a barrier of fx_staples' first iteration
-template <int N, bool SYNC, bool SHARE, class SRC, class SKIP, class VISIT>
-__device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shared<N>* sh, int lane, const CfgDesc& c, int s, int mu, unsigned eb, fx_guard& g,
-                                           SKIP&& skip, VISIT&& visit, int q0 = 0, int q1 = 6) {
+template <int N, bool SYNC, bool SHARE, class SRC, class VISIT>
+__device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shared<N>* sh, int lane, const CfgDesc& c, int s,
+                                           int mu, unsigned eb, fx_guard& g, VISIT&& visit, int q0 = 0, int q1 = 6) {
     const int s_mp = fwd(c, eb, s, mu);
     const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
     const long long half = fx_round();
@@ -323,7 +323,6 @@ __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shar
         const bool back = q & 1;
         const int nu = (mu + 1 + (q >> 1)) & 3;
         if (SYNC) __syncthreads();
-        if (skip(nu)) continue;
         const int s_nm = bwd(c, eb, s, nu);
         const int sb = back ? s_nm : fwd(c, eb, s, nu);
         const int sv = back ? s_nm : s_mp;

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ Ba
     {
         matq<3> sig;
         fx_zero(sig);
-        fx_staples<3, true, false>(sig, src, nullptr, 0, c, s, mu, eb, g, [](int) { return false; }, [](int, int, const matq<3>&) {});
+        fx_staples<3, true, false>(sig, src, nullptr, 0, c, s, mu, eb, g, [](int, int, const matq<3>&) {});
         if (!valid) return;
         matx<3> u, sx;
         matq<3> om;

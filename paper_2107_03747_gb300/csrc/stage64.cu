@@ -14,13 +14,13 @@ template <int STAGE, int MODE, int CAP, bool WIDE>
 void launch_cap(const Batch& B, const double* w_in, double* w_out, double* acc, double* clov, cudaStream_t st, int grid) {
     const int g = (grid > 0 && grid < B.nblk) ? grid : B.nblk;
     if constexpr (CAP == kMaxCfg) {
-        k_stage64<STAGE, MODE, kMaxCfg, WIDE><<<g, WIDE ? 384 : 128, 0, st>>>(B, w_in, w_out, acc, clov);
+        k_stage64<STAGE, MODE, kMaxCfg, WIDE><<<g, stage64_threads(MODE, WIDE), 0, st>>>(B, w_in, w_out, acc, clov);
     } else {
         BatchT<CAP> b;
         b.ncfg = B.ncfg;
         b.nblk = B.nblk;
         for (int i = 0; i < B.ncfg; ++i) b.c[i] = B.c[i];
-        k_stage64<STAGE, MODE, CAP, WIDE><<<g, WIDE ? 384 : 128, 0, st>>>(b, w_in, w_out, acc, clov);
+        k_stage64<STAGE, MODE, CAP, WIDE><<<g, stage64_threads(MODE, WIDE), 0, st>>>(b, w_in, w_out, acc, clov);
     }
 }
 

@@ -59,7 +59,6 @@ __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c
     for (int dn = dn0; dn < dn1; ++dn) {
         const int nu = (mu + dn) & 3;
         const bool clover = MODE != 0 && c_clover_owner[mu][nu];
-        if (MODE == 2 && !clover) continue;
         const int s_nm = bwd(c, eb, s, nu);
         const int k = c.tw[mu * 4 + nu];
         double zr = 1.0, zi = 0.0;
@@ -109,16 +108,20 @@ __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c
 }
 
 // One thread per link; a block covers 32 sites x 4 directions, warps grouped by mu.  MODE as in k_stage:
-// 0 the stage, 1 the stage and the clover halves of the input field, 2 the halves only.
+// 0 the stage, 1 the stage and the clover halves of the input field, 2 the halves only (three warps with two planes
+// each, c_half; WIDE: six with one).
 //
 // WIDE: three threads per link, one for each direction nu, whose staple sums meet in shared memory (whole numbers:
 // the result is the same to the bit) before the first goes on with the link.  For launches that leave most of
 // the chip idle (launch_m in stage64.cu).
+constexpr int stage64_threads(int mode, bool wide) { return mode == 2 ? (wide ? 192 : 96) : wide ? 384 : 128; }
 template <int STAGE, int MODE, int CAP, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? 384 : 128, WIDE ? 1 : MODE == 0 ? 3 : 2)
+__global__ void __launch_bounds__(stage64_threads(MODE, WIDE), WIDE ? 1 : MODE == 0 ? 3 : MODE == 1 ? 2 : 4)
 k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
           double* __restrict__ acc, double* __restrict__ clov) {
-    const int mu = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31, part = threadIdx.x >> 7;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int mu = warp & 3;
+    const int part = MODE == 2 ? 0 : warp >> 2;
     // the links shared by the block's warps; WIDE: then the staple sums of its second and third part
     __shared__ union {
         fx_shared<3> links;
@@ -149,15 +152,26 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
         if (MODE != 0) fx_zero(kk);
         __syncthreads();  // the block before is done with the shared memory
 #pragma unroll 1
-        for (int m = mu + 4 * part; m < 8; m += WIDE ? 12 : 4) {
+        for (int m = warp; m < 8; m += (int)blockDim.x >> 5) {
             fx_guard gl;
-            fx_take_matrix<3>(u, src, mu, m < 4 ? s : bwd(c, eb, s, mu), false, gl);
+            fx_take_matrix<3>(u, src, m & 3, m < 4 ? s : bwd(c, eb, s, m & 3), false, gl);
             fx_share<3>(sm.links, m, lane, u, gl);
         }
-        fx_staples<3, true, true>(sig, src, &sm.links, lane, c, s, mu, eb, g, [&](int nu) { return MODE == 2 && !c_clover_owner[mu][nu]; },
-            [&](int back, int nu, const matq<3>& sum) {
+#pragma unroll 1
+        for (int it = 0; it < (MODE == 2 && !WIDE ? 2 : 1); ++it) {
+            int q0 = WIDE ? 2 * part : 0, q1 = WIDE ? 2 * part + 2 : 6;
+            if (MODE == 2) {
+                const int e = WIDE ? warp : 2 * warp + it;
+                mu = c_half[e][0];
+                q0 = 2 * ((c_half[e][1] - mu - 1) & 3);
+                q1 = q0 + 2;
+                fx_zero(sig);
+                fx_zero(kk);
+                g = fx_guard{};
+            }
+            fx_staples<3, true, true>(sig, src, &sm.links, lane, c, s, mu, eb, g, [&](int back, int nu, const matq<3>& sum) {
                 if (!valid || MODE == 0) return;
-                if (!c_clover_owner[mu][nu]) {
+                if (MODE == 1 && !c_clover_owner[mu][nu]) {
                     if (back) kk = sum;
                     return;
                 }
@@ -201,11 +215,16 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 fx_mul_nn<3>(t, kx, u);
                 fx_store_ah(cb + (size_t)(pl * 2 + 1) * 9 * Vp, Vp, fwd(c, eb, s, mu), t, unit);
                 kk = sum;
-            },
-            WIDE ? 2 * part : 0, WIDE ? 2 * part + 2 : 6);
-        fx_shared_link<3>(u, sm.links, mu, lane);
+            }, q0, q1);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) g.top2 |= sm.links.bad[m][lane];
+            for (int m = 0; m < 8; ++m) g.top2 |= sm.links.bad[m][lane];
+            if (MODE == 2 && valid && g.bad()) {
+                alg8<double> z;
+                native_force64<MODE>(z, c, base, cb, s, mu, eb, q0 / 2 + 1, q0 / 2 + 2);
+            }
+        }
+        if (MODE == 2) continue;
+        fx_shared_link<3>(u, sm.links, mu, lane);
         if constexpr (WIDE && MODE != 2) {
             const int lt = threadIdx.x & 127;
             __syncthreads();  // the links have been read: their place takes the sums
@@ -231,13 +250,6 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
             fx_check<3, 29>(sig, g);
         }
         if (!valid) continue;
-        if (MODE == 2) {
-            if (g.bad()) {
-                alg8<double> z;
-                native_force64<MODE>(z, c, base, cb, s, mu, eb, WIDE ? 1 + part : 1, WIDE ? 2 + part : 4);
-            }
-            continue;
-        }
         // Omega = U_mu(n) Sigma (units 2^-56), Z = -P_ta(Omega)
         alg8<double> x, z;
         {

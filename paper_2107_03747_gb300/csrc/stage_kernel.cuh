@@ -118,10 +118,15 @@ __device__ __forceinline__ void bar_arrive(int id, int nthreads) {
 __device__ __forceinline__ void bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-// the measured stage 1 (MODE 1: clover halves too) needs more registers: at most 4 blocks per SM
+// the measured stage 1 (MODE 1: clover halves too) needs more registers: at most 4 blocks per SM; mode 2 has blocks of
+// three warps (c_half)
+template <int TILE, int MODE>
+constexpr int stage_threads() {
+    return MODE == 2 ? 96 : 4 * StageTile<TILE>::spb;
+}
 template <int P, int TILE, int MODE>
 constexpr int stage_min_blocks() {
-    return (MODE != 0 && StageTile<TILE>::minb32 > 4) ? 4 : StageTile<TILE>::minb32;
+    return MODE == 2 ? 5 : (MODE != 0 && StageTile<TILE>::minb32 > 4) ? 4 : StageTile<TILE>::minb32;
 }
 
 // MODE 0: the RK3 stage.  MODE 1: the stage, and from the same staples of the input field the
@@ -134,7 +139,7 @@ constexpr int stage_min_blocks() {
 // Thread (n, mu) writes D1 - D1^+ to site n and D2 - D2^+ to site n + mu for the planes its warp
 // builds (c_clover_owner), plus 3 - Re Tr(U F) (the twisted plaquette at n).
 template <int P, int STAGE, int MODE, int TILE, int CAP>
-__global__ void __launch_bounds__(4 * StageTile<TILE>::spb, (stage_min_blocks<P, TILE, MODE>()))
+__global__ void __launch_bounds__((stage_threads<TILE, MODE>()), (stage_min_blocks<P, TILE, MODE>()))
 k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __restrict__ w_in,
         typename Store<P>::T* __restrict__ w_out, typename Store<P>::T* __restrict__ acc,
         typename Store<P>::T* __restrict__ clov, int reunit) {
@@ -144,7 +149,7 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
     constexpr int SPB = StageTile<TILE>::spb;
     static_assert(P != P64, "FP64: stage64.cuh");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int mu = warp & 3;
+    const int dir = warp & 3;  // the warp's link direction (mode 2: c_half)
     const int row = warp >> 2;  // which 32-site row of the block
     // tile 3 (FP32 forms, unmeasured stages): corners shared in pairs; every lane of the block's four
     // warps takes part in the named barriers, lanes past the configuration's end on site 0 with
@@ -198,14 +203,16 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
         };
         mat3<T> sig, a, b, t;
         auto link_body = [&]() {
-        const int s_mp = fwd(c, eb, s, mu);
-        const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
+        const int s_dir = fwd(c, eb, s, dir);
+        const bool at_dir0 = (eb >> dir) & 1u;
         if (MODE != 2) set_zero(sig);
 #pragma unroll 1
-        for (int dn = 1; dn < 4; ++dn) {
-            const int nu = PAIR ? (int)c_pair_nu[mu][dn - 1] : (mu + dn) & 3;
-            const bool clover = MODE != 0 && c_clover_owner[mu][nu];
-            if (MODE == 2 && !clover) continue;
+        for (int dn = 1; dn < (MODE == 2 ? 3 : 4); ++dn) {
+            const int mu = MODE == 2 ? (int)c_half[2 * warp + dn - 1][0] : dir;
+            const int nu = MODE == 2 ? (int)c_half[2 * warp + dn - 1][1] : PAIR ? (int)c_pair_nu[mu][dn - 1] : (mu + dn) & 3;
+            const bool clover = MODE == 2 || (MODE == 1 && c_clover_owner[mu][nu]);
+            const int s_mp = MODE == 2 ? fwd(c, eb, s, mu) : s_dir;
+            const bool at_mu0 = MODE == 2 ? (bool)((eb >> mu) & 1u) : at_dir0;  // x_mu = 0: the twisted plaquettes' corner row
             const int s_nm = bwd(c, eb, s, nu);
             const int s_mp_nm = fwd(c, eb, s_nm, mu);  // x_mu(n - nu) = x_mu(n)
             const int k = c.tw[mu * 4 + nu];
@@ -292,6 +299,7 @@ k_stage(const __grid_constant__ BatchT<CAP> B, const typename Store<P>::T* __res
         }
         if (MODE == 2) return;
         // Omega = U_mu(n) Sigma, Z = -P_ta(Omega)
+        const int mu = dir;
         mat3<T> u;
         link(mu, s, u);
         mul_nn_ah(t, u, sig);
@@ -334,17 +342,16 @@ template <int P, int STAGE, int MODE, int TILE, int CAP>
 static void launch_cap(const Batch& B, const void* w_in, void* w_out, void* acc, void* clov, int reunit,
                        cudaStream_t st, int grid) {
     using T = typename Store<P>::T;
-    constexpr int SPB = StageTile<TILE>::spb;
     const int g = (grid > 0 && grid < B.nblk) ? grid : B.nblk;
     if constexpr (CAP == kMaxCfg) {
-        k_stage<P, STAGE, MODE, TILE, kMaxCfg><<<g, 4 * SPB, 0, st>>>(B, (const T*)w_in, (T*)w_out, (T*)acc,
+        k_stage<P, STAGE, MODE, TILE, kMaxCfg><<<g, stage_threads<TILE, MODE>(), 0, st>>>(B, (const T*)w_in, (T*)w_out, (T*)acc,
                                                                      (T*)clov, reunit);
     } else {
         BatchT<CAP> b;
         b.ncfg = B.ncfg;
         b.nblk = B.nblk;
         for (int i = 0; i < B.ncfg; ++i) b.c[i] = B.c[i];
-        k_stage<P, STAGE, MODE, TILE, CAP><<<g, 4 * SPB, 0, st>>>(b, (const T*)w_in, (T*)w_out, (T*)acc,
+        k_stage<P, STAGE, MODE, TILE, CAP><<<g, stage_threads<TILE, MODE>(), 0, st>>>(b, (const T*)w_in, (T*)w_out, (T*)acc,
                                                                  (T*)clov, reunit);
     }
 }

@@ -497,7 +497,7 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
     {
         matq<N> sig, om;
         fx_zero(sig);
-        fx_staples<N, true, false>(sig, src, nullptr, 0, c, s, mu, eb, g, [](int) { return false; }, [](int, int, const matq<N>&) {});
+        fx_staples<N, true, false>(sig, src, nullptr, 0, c, s, mu, eb, g, [](int, int, const matq<N>&) {});
         if (!valid) return;
         // Omega = U Sigma (units 2^-56); Z = -P_ta(Omega) = -(Omega - Omega^+)/2 + tr(Omega - Omega^+)/(2N)
         matx<N> sx;

@@ -468,10 +468,16 @@ __device__ __forceinline__ unsigned fx_exp_m1<4>(matx<4>& o, const matN<4>& X, f
     return up;
 }
 
+// Whether the block's warps share operands: splitting a link costs 14 instructions per real entry, a shared one a
+// 16-byte load per entry.  SU(3) 3 % and SU(4) 8 % faster (1103 -> 1065 us, 4.83 -> 4.44 ms for the case below),
+// SU(2) 0.6 % slower.
+template <int N>
+constexpr bool kSunShares = N > 2;
+
 // one RK3 stage for SU(N); block = 4 warps (one per direction) x 32 sites.  Matrix products in fixed point
 // on the integer pipe (fixed.cuh), scalars in FP64, as the SU(3) kernels of stage64.cuh; all of it in FP64 kept
 // that pipe 90-96 % busy.  Two steps and a measurement of 8 x 8x8x16x16 in SU(2): 4.08 ms before, 1.51 now; one
-// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.83 now.
+// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.44 now.
 template <int N, int STAGE, int CAP>
 __global__ void __launch_bounds__(128, N == 4 ? 2 : 3)
 k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
@@ -491,18 +497,37 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
     const double* base = w_in + c.w_off;
     fx_guard g;
     SunSrc<N> src{reinterpret_cast<const double2*>(base), Vp};
+    // the links at n and one step back in each direction, shared by the block's warps (kSunShares)
+    constexpr bool SHARE = kSunShares<N>;
+    extern __shared__ __align__(16) unsigned char s_links[];
+    fx_shared<N>& links = *reinterpret_cast<fx_shared<N>*>(s_links);
     matx<N> u;
+    if (SHARE) {
+#pragma unroll 1
+        for (int m = mu; m < 8; m += 4) {
+            fx_guard gl;
+            fx_take_matrix<N>(u, src, mu, m < 4 ? s : bwd(c, eb, s, mu), false, gl);
+            fx_share<N>(links, m, lane, u, gl);
+        }
+    }
+    auto own_link = [&]() {
+        if (SHARE) fx_shared_link<N>(u, links, mu, lane);
+        else fx_take_matrix<N>(u, src, mu, s, false, g);
+    };
     matN<N> X;
     double x[N * N];  // Z, then X: diagonal imaginary parts, then (re, im) above the diagonal
     {
         matq<N> sig, om;
         fx_zero(sig);
-        fx_staples<N, true, false>(sig, src, nullptr, 0, c, s, mu, eb, g, [](int, int, const matq<N>&) {});
+        fx_staples<N, true, SHARE>(sig, src, &links, lane, c, s, mu, eb, g, [](int, int, const matq<N>&) {});
         if (!valid) return;
+        if (SHARE)
+#pragma unroll
+            for (int m = 0; m < 8; ++m) g.top2 |= links.bad[m][lane];
         // Omega = U Sigma (units 2^-56); Z = -P_ta(Omega) = -(Omega - Omega^+)/2 + tr(Omega - Omega^+)/(2N)
         matx<N> sx;
         fx_operand_wide<N, 2>(sx, sig);
-        fx_take_matrix<N>(u, src, mu, s, false, g);
+        own_link();
         fx_mul_nn<N>(om, u, sx);
         long long tr = 0;
 #pragma unroll
@@ -570,6 +595,7 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
     } else {
         // W' = W + (exp(X) - 1) W, rounded once onto W
         matq<N> d;
+        if (SHARE) own_link();
         fx_mul_nn<N>(d, ex, u);
         const double unit = fx_unit(up);
 #pragma unroll
@@ -856,9 +882,15 @@ BatchT<CAP> shrink(const Batch& B) {
 template <int N, int CAP>
 void sun_stage_cap(int stage, const Batch& B, const double* w_in, double* w_out, double* acc, cudaStream_t st) {
     const BatchT<CAP> b = shrink<CAP>(B);
-    if (stage == 1) k_sun_stage<N, 1, CAP><<<B.nblk, 128, 0, st>>>(b, w_in, w_out, acc);
-    else if (stage == 2) k_sun_stage<N, 2, CAP><<<B.nblk, 128, 0, st>>>(b, w_in, w_out, acc);
-    else k_sun_stage<N, 3, CAP><<<B.nblk, 128, 0, st>>>(b, w_in, w_out, acc);
+    auto launch = [&](auto kernel) {
+        constexpr int bytes = kSunShares<N> ? (int)sizeof(fx_shared<N>) : 0;
+        // a failure is the launch's to report
+        if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        kernel<<<B.nblk, 128, bytes, st>>>(b, w_in, w_out, acc);
+    };
+    if (stage == 1) launch(k_sun_stage<N, 1, CAP>);
+    else if (stage == 2) launch(k_sun_stage<N, 2, CAP>);
+    else launch(k_sun_stage<N, 3, CAP>);
 }
 
 template <int N, int CAP>

@@ -173,27 +173,35 @@ __device__ __forceinline__ quat su2_block(const mat3<double>& w, int i, int j) {
             w.e[i][i].im - w.e[j][j].im};
 }
 
+// R as operands: rows (r00, r01) and (-r01^*, r00^*) and their negatives.  |R| = 1 to FP64 rounding, as x is
+// finite where this is used, so no entry needs a check.
+struct rot_fx {
+    vecx<2> i, ni, j, nj;
+};
+__device__ __forceinline__ void take_rotation(rot_fx& o, const rot2& R) {
+    fx_guard g;
+    fx_take(R.a.re, o.i.rh[0], o.i.rl[0], g);
+    fx_take(R.a.im, o.i.ih[0], o.i.il[0], g);
+    fx_take(R.b.re, o.i.rh[1], o.i.rl[1], g);
+    fx_take(R.b.im, o.i.ih[1], o.i.il[1], g);
+    o.ni = fx_negated(o.i);
+    o.j.rh[0] = o.ni.rh[1]; o.j.rl[0] = o.ni.rl[1]; o.j.ih[0] = o.i.ih[1]; o.j.il[0] = o.i.il[1];
+    o.j.rh[1] = o.i.rh[0]; o.j.rl[1] = o.i.rl[0]; o.j.ih[1] = o.ni.ih[0]; o.j.il[1] = o.ni.il[0];
+    o.nj = fx_negated(o.j);
+}
+
 // rows i, j of the link by R, in fixed point: rows that a later rotation reads are taken back as
 // operands, finished rows stay as sums
 template <bool KEEP_I, bool KEEP_J>
-__device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j, const rot2& R, fx_guard& g) {
+__device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j, const rot_fx& R) {
     const long long half = fx_round();
-    vecx<2> ri, rj;  // (r00, r01) and (-r01^*, r00^*)
-    fx_take(R.a.re, ri.rh[0], ri.rl[0], g);
-    fx_take(R.a.im, ri.ih[0], ri.il[0], g);
-    fx_take(R.b.re, ri.rh[1], ri.rl[1], g);
-    fx_take(R.b.im, ri.ih[1], ri.il[1], g);
-    const vecx<2> n = fx_negated(ri);
-    rj.rh[0] = n.rh[1]; rj.rl[0] = n.rl[1]; rj.ih[0] = ri.ih[1]; rj.il[0] = ri.il[1];
-    rj.rh[1] = ri.rh[0]; rj.rl[1] = ri.rl[0]; rj.ih[1] = n.ih[0]; rj.il[1] = n.il[0];
-    const vecx<2> nj = fx_negated(rj);
 #pragma unroll
     for (int col = 0; col < 3; ++col) {
         vecx<2> p;
         p.rh[0] = u.rh[i][col]; p.rl[0] = u.rl[i][col]; p.ih[0] = u.ih[i][col]; p.il[0] = u.il[i][col];
         p.rh[1] = u.rh[j][col]; p.rl[1] = u.rl[j][col]; p.ih[1] = u.ih[j][col]; p.il[1] = u.il[j][col];
         long long re = 0, im = 0;
-        fx_dot<2, false>(re, im, ri, n, p, half);
+        fx_dot<2, false>(re, im, R.i, R.ni, p, half);
         if (KEEP_I) {
             fx_split<0>(re, u.rh[i][col], u.rl[i][col]);
             fx_split<0>(im, u.ih[i][col], u.il[i][col]);
@@ -202,7 +210,7 @@ __device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j
             out.im[i][col] = im;
         }
         re = im = 0;
-        fx_dot<2, false>(re, im, rj, nj, p, half);
+        fx_dot<2, false>(re, im, R.j, R.nj, p, half);
         if (KEEP_J) {
             fx_split<0>(re, u.rh[j][col], u.rl[j][col]);
             fx_split<0>(im, u.ih[j][col], u.il[j][col]);
@@ -213,10 +221,64 @@ __device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j
     }
 }
 
-// Matrix products of the staples, Omega and the rotations of U run in fixed point on the integer pipe
-// (fixed.cuh), the SU(2) blocks and draws in FP64, and an over-relaxation takes (v^+)^2 from x with one
-// division: about 210 FP64 instructions instead of 2,200, which kept the FP64 pipe 94 % busy.
-// One hybrid sweep (1 heat-bath, 12 over-relaxation) of 256 x 4x4x12x12: 114.9 ms before, 33.2 now.
+// entry (i, col) and/or (j, col) of W by R.  W's parts are checked to be below kWideW (six unitary matrices sum to
+// 6 at most); the rotations keep the norm of the three entries of a column, so a part stays below
+// sqrt(6) 6.25 = 15.4, hi below 2^31 and the sums of fx_dot below 2^62.4.
+constexpr int kWideW = 25 << 22;  // 6.25 in the top word of a sum in units 2^-56
+template <bool I, bool J>
+__device__ __forceinline__ void fx_rotate_entry(matq<3>& w, int i, int j, int col, const rot_fx& R) {
+    const long long half = fx_round();
+    vecx<2> p;
+    fx_split<0>(w.re[i][col], p.rh[0], p.rl[0]);
+    fx_split<0>(w.im[i][col], p.ih[0], p.il[0]);
+    fx_split<0>(w.re[j][col], p.rh[1], p.rl[1]);
+    fx_split<0>(w.im[j][col], p.ih[1], p.il[1]);
+    if (I) {
+        w.re[i][col] = w.im[i][col] = 0;
+        fx_dot<2, false>(w.re[i][col], w.im[i][col], R.i, R.ni, p, half);
+    }
+    if (J) {
+        w.re[j][col] = w.im[j][col] = 0;
+        fx_dot<2, false>(w.re[j][col], w.im[j][col], R.j, R.nj, p, half);
+    }
+}
+
+// the block of W, a sum before it is rounded to FP64
+__device__ __forceinline__ quat su2_block(const matq<3>& w, int i, int j) {
+    return {(double)(w.re[i][i] + w.re[j][j]), (double)(w.im[i][j] + w.im[j][i]), (double)(w.re[i][j] - w.re[j][i]),
+            (double)(w.im[i][i] - w.im[j][j])};
+}
+
+// The whole update in FP64, for links whose staples leave the range of fixed.cuh
+template <int OVERRELAX>
+__device__ __forceinline__ void native_update(double* __restrict__ base, int Vp, const CfgDesc& c, int s, unsigned eb, int mu,
+                                              double beta, uint64_t key, uint64_t c0) {
+    mat3<double> wm, un;
+    native_omega(wm, base, Vp, c, s, eb, mu);
+    Store<P64>::load(base + (size_t)mu * 18 * Vp, Vp, s, un);
+#pragma unroll 1
+    for (int sub = 0; sub < 3; ++sub) {
+        const int i = sub >> 1, j = sub == 0 ? 1 : 2;
+        const rot2 R = draw_rotation<OVERRELAX>(su2_block(wm, i, j), 1.0, beta, key, c0 + sub * kSlots);
+        for (int col = 0; col < 3; ++col) {
+            cx<double> p = wm.e[i][col], q = wm.e[j][col];
+            wm.e[i][col] = rot_i(R, p, q);
+            wm.e[j][col] = rot_j(R, p, q);
+            p = un.e[i][col], q = un.e[j][col];
+            un.e[i][col] = rot_i(R, p, q);
+            un.e[j][col] = rot_j(R, p, q);
+        }
+    }
+    Store<P64>::store(base + (size_t)mu * 18 * Vp, Vp, s, un);
+}
+
+// Staples, W and the rotations of W and U run in fixed point on the integer pipe (fixed.cuh); FP64 keeps the
+// SU(2) blocks' direction (an over-relaxation takes (v^+)^2 from x with one division), the heat-bath's draws and the
+// conversion of the result: about 130 FP64 instructions instead of 2,200, which kept the FP64 pipe 94 % busy.
+// W rotated in FP64 put 210 there, in three chains that nothing overlaps.
+// One hybrid sweep (1 heat-bath, 12 over-relaxation) of 256 x 4x4x12x12: 114.9 ms in FP64, 33.2 with W rotated in
+// FP64, 31.7 now; of 60 such fields 9.93 -> 9.06, of 8 3.76 -> 3.47.  The integer pipe is about 66 % busy; with 168 registers an SM holds
+// 12 warps, and 4 blocks of it spill (35.8 ms).
 template <int OVERRELAX, int CAP>
 __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ BatchT<CAP> B, double* __restrict__ w,
                                                       int mu, int parity, double beta, uint64_t seed, uint64_t sweep) {
@@ -244,70 +306,59 @@ __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ Ba
 
     fx_guard g;
     Su3Src src{base, Vp};
-    mat3<double> wm;
+    matq<3> om;  // W, in units 2^-56: the rotations depend on its direction only, but for the heat-bath's alpha
     {
         matq<3> sig;
         fx_zero(sig);
         fx_staples<3, true, false>(sig, src, nullptr, 0, c, s, mu, eb, g, [](int, int, const matq<3>&) {});
         if (!valid) return;
         matx<3> u, sx;
-        matq<3> om;
         fx_operand_wide<3, 2>(sx, sig);
         fx_take_matrix<3>(u, src, mu, s, false, g);
         fx_mul_nn<3>(om, u, sx);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) wm.e[i][k] = {(double)om.re[i][k], (double)om.im[i][k]};
     }
-    double unit = 0x1p-56;  // of W: the rotations depend on its direction only, but for the heat-bath's alpha
-    if (g.bad()) {
-        native_omega(wm, base, Vp, c, s, eb, mu);
-        unit = 1.0;
-    }
+    unsigned wide = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            wide = max(wide, (unsigned)((int)(om.re[i][k] >> 32) + kWideW));
+            wide = max(wide, (unsigned)((int)(om.im[i][k] >> 32) + kWideW));
+        }
     const uint64_t key = hash64(seed, (uint64_t)ci);
     const uint64_t c0 = (((uint64_t)sweep * 4 + (uint64_t)mu) * (uint64_t)c.V + (uint64_t)s) * 3 * kSlots;
+    if (g.bad() || wide >= 2u * kWideW) {
+        native_update<OVERRELAX>(base, Vp, c, s, eb, mu, beta, key, c0);
+        return;
+    }
     // the three subgroups (0,1), (0,2), (1,2), each on W after the ones before it; only the entries
     // that a later block reads are rotated
-    const rot2 R0 = draw_rotation<OVERRELAX>(su2_block(wm, 0, 1), unit, beta, key, c0);
-    {
-        const cx<double> p1 = wm.e[0][1], p2 = wm.e[0][2];
-#pragma unroll
-        for (int col = 0; col < 3; ++col) wm.e[0][col] = rot_i(R0, wm.e[0][col], wm.e[1][col]);
-        wm.e[1][1] = rot_j(R0, p1, wm.e[1][1]);
-        wm.e[1][2] = rot_j(R0, p2, wm.e[1][2]);
-    }
-    const rot2 R1 = draw_rotation<OVERRELAX>(su2_block(wm, 0, 2), unit, beta, key, c0 + kSlots);
-    wm.e[2][1] = rot_j(R1, wm.e[0][1], wm.e[2][1]);
-    wm.e[2][2] = rot_j(R1, wm.e[0][2], wm.e[2][2]);
-    const rot2 R2 = draw_rotation<OVERRELAX>(su2_block(wm, 1, 2), unit, beta, key, c0 + 2 * kSlots);
-
+    constexpr double kUnit = 0x1p-56;
     matx<3> u;
     matq<3> out;
+    rot_fx R;
+    take_rotation(R, draw_rotation<OVERRELAX>(su2_block(om, 0, 1), kUnit, beta, key, c0));
+    fx_rotate_entry<true, false>(om, 0, 1, 0, R);
+    fx_rotate_entry<true, true>(om, 0, 1, 1, R);
+    fx_rotate_entry<true, true>(om, 0, 1, 2, R);
+    // U is taken in a second time rather than held over the first draw (36 registers: 31.8 instead of 31.7 ms for
+    // the sweep below, 3.53 instead of 3.37 for 8 fields); the opaque copy keeps the compiler from merging the two
+    int dir = mu;
+    asm volatile("" : "+r"(dir));
+    fx_take_matrix<3>(u, src, dir, s, false, g);
+    fx_rotate<true, true>(out, u, 0, 1, R);
+    take_rotation(R, draw_rotation<OVERRELAX>(su2_block(om, 0, 2), kUnit, beta, key, c0 + kSlots));
+    fx_rotate_entry<false, true>(om, 0, 2, 1, R);
+    fx_rotate_entry<false, true>(om, 0, 2, 2, R);
+    fx_rotate<false, true>(out, u, 0, 2, R);
+    take_rotation(R, draw_rotation<OVERRELAX>(su2_block(om, 1, 2), kUnit, beta, key, c0 + 2 * kSlots));
+    fx_rotate<false, false>(out, u, 1, 2, R);
+
     mat3<double> un;
-    fx_take_matrix<3>(u, src, mu, s, false, g);
-    fx_rotate<true, true>(out, u, 0, 1, R0, g);
-    fx_rotate<false, true>(out, u, 0, 2, R1, g);
-    fx_rotate<false, false>(out, u, 1, 2, R2, g);
-    if (g.bad()) {
-        Store<P64>::load(base + (size_t)mu * 18 * Vp, Vp, s, un);
-        auto rot = [&](int i, int k, const rot2& R) {
 #pragma unroll
-            for (int col = 0; col < 3; ++col) {
-                const cx<double> p = un.e[i][col], q = un.e[k][col];
-                un.e[i][col] = rot_i(R, p, q);
-                un.e[k][col] = rot_j(R, p, q);
-            }
-        };
-        rot(0, 1, R0);
-        rot(0, 2, R1);
-        rot(1, 2, R2);
-    } else {
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) un.e[i][k] = {fx_value(out.re[i][k]), fx_value(out.im[i][k])};
-    }
+        for (int k = 0; k < 3; ++k) un.e[i][k] = {fx_value(out.re[i][k]), fx_value(out.im[i][k])};
     Store<P64>::store(base + (size_t)mu * 18 * Vp, Vp, s, un);
 }
 

@@ -42,6 +42,11 @@ def edge_field(kind, N=3, L=L, amp=0.7):
         return u
     if kind == "all_large":
         return 3.0 * u
+    if kind == "wide":  # links of one direction far from unitary, every entry and staple sum within its bound, W not
+        v = np.zeros_like(u)
+        v[..., range(N), range(N)] = 1.0
+        v[:, :, :, :, 0] = rng.choice([-1.0, 1.0], (N, N)) + 1j * rng.choice([-1.0, 1.0], (N, N))
+        return v
     if kind == "just_in":  # at the bound of a link entry
         v = np.zeros_like(u)
         v[..., range(N), range(N)] = 1.0 + 2.0 ** -11
@@ -99,7 +104,7 @@ def test_one_bad_link_stays_local(tgf):
     assert np.abs(got - ref)[~bad].max() <= 100 * U
 
 
-@pytest.mark.parametrize("kind", ["su", "unit", "some_large", "all_large"])
+@pytest.mark.parametrize("kind", ["su", "unit", "some_large", "all_large", "wide"])
 @pytest.mark.parametrize("n_or", [0, 2])
 def test_monte_carlo_matches_the_oracle_at_the_edges_of_the_range(tgf, kind, n_or):
     # bar of the Monte Carlo parity tests: rounding amplified by the division by k, 1e-10 on the links

@@ -102,8 +102,8 @@ typedef enum {
                                      such check is not finite                                       */
 /* Launch tuning of tgf_flow (results are bitwise the same for every setting; the tuner of the
  * Python package times them per workload): TGF_TUNE_GRID(k), k = 1..15, launches the stage
- * kernels as a persistent grid of k x (number of SMs) x (resident blocks per SM: 4 in FP32,
- * 2 in FP64) that loops over the tiles, instead of one block per tile (k = 0);
+ * kernels as a persistent grid of k x (number of SMs) x (4 blocks in FP32, 2 in FP64) that loops
+ * over the tiles, instead of one block per tile (k = 0);
  * TGF_TUNE_SIZE_ORDER orders the configurations of each launch by size, largest first. */
 #define TGF_TUNE_GRID(k) (((unsigned)(k) & 0xFu) << 8)
 #define TGF_TUNE_SIZE_ORDER (1u << 12)

@@ -177,7 +177,8 @@ k_reduce(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ parti
 // fixed order.  A slab is cut into chunks of kSliceSites sites, one block and one site per thread each
 // (the launch descriptor has L[dir] slice_chunks(n_slab) blocks per configuration), so that a few long slabs still
 // fill the chip: with one block per slab, 72 slabs of 5184 sites left half the SMs idle and took 75 us, now 29 and 4
-// for the sums (the halves' 161 MB at 6.7 TB/s take 24); tgf_measure_slices of 2 x 12x12x36x36 in FP32 183 -> 139 us.
+// for the sums (the halves' 161 MB at 6.7 TB/s take 24); tgf_measure_slices of 2 x 12x12x36x36 in FP32 183 -> 139 us
+// (127 with the halves of planes.cuh).
 // A slab of one chunk is finished here; the
 // others leave a partial sum per block (x_off: the configuration's first one) for k_slice_reduce.
 // q_out[cfg_index * q_stride + x] with cfg_index = c.o_off.

@@ -6,8 +6,9 @@
 // quarter), and nothing else of the chip was in use.  Here that pipe carries about 115 instructions (7,200
 // cycles) and the integer pipe 13 products (4,900 IMAD.WIDE of 4 cycles) and the splitting of the operands:
 // 34,000 cycles, the multiply pipe 65 % busy.  4 steps of 4 x 8x8x24x24, measured each step: 23.8 ms before,
-// 8.6 with the products in fixed point, 7.8 with the exponential (fx_exp_su3) as well; one measurement of
-// 4 x 7x7x21x21: 693 us before, 312 now; 3 steps of 4x4x12x12 (latency): 698 us before, 295 now.
+// 8.6 with the products in fixed point, 7.8 with the exponential (fx_exp_su3) as well, 7.6 with the block's
+// links taken in once and shared; one measurement of 4 x 7x7x21x21: 693 us before, 272 now; 3 steps of
+// 4x4x12x12 (latency): 696 us before, 281 now.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -57,8 +57,8 @@ __device__ __forceinline__ void reunitarize(mat3<T>& u) {
 }
 
 // Launch tiles of the stage kernel (chosen per workload by the launch tuner, flag TGF_TUNE_TILE):
-//   0  32 sites per block, one warp per direction, 4 resident blocks per SM in the FP32 forms
-//      (at most 128 registers per thread), 2 in FP64
+//   0  32 sites per block, one warp per direction, 4 resident blocks per SM (at most 128 registers
+//      per thread)
 //   1  64 sites per block, two warps per direction (a block spans two 32-site rows), 2 resident
 //      blocks of 256 threads per SM (at most 128 registers)
 //   2  32 sites per block as a 4 x 2 x 2 x 2 hypercube (x0 x1 x2 x3) instead of 32 consecutive
@@ -69,7 +69,7 @@ __device__ __forceinline__ void reunitarize(mat3<T>& u) {
 //      corners T_ab in pairs through shared memory (below)
 //   4  as 0 with a tighter register cap in the unmeasured stages: 5 resident blocks per SM (at
 //      most 102 registers; the measured stage 1 keeps 4), more warps to cover latency
-// Tiles 1 to 4 exist for the FP32 forms only.  Tiles 0, 1, 2 and 4 compute the same flow bit for
+// FP64 has a kernel of its own (stage64.cuh).  Tiles 0, 1, 2 and 4 compute the same flow bit for
 // bit; tile 3 forms the shared staples as (Z T_ba)^+ U^+ instead of Z* T_ab U^+, equal up to
 // rounding.
 template <int TILE>

@@ -476,8 +476,8 @@ constexpr bool kSunShares = N > 2;
 
 // one RK3 stage for SU(N); block = 4 warps (one per direction) x 32 sites.  Matrix products in fixed point
 // on the integer pipe (fixed.cuh), scalars in FP64, as the SU(3) kernels of stage64.cuh; all of it in FP64 kept
-// that pipe 90-96 % busy.  Two steps and a measurement of 8 x 8x8x16x16 in SU(2): 4.08 ms before, 1.51 now; one
-// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.44 now.
+// that pipe 90-96 % busy.  Two steps and a measurement of 8 x 8x8x16x16 in SU(2): 4.08 ms before, 1.45 now; one
+// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.30 now.
 template <int N, int STAGE, int CAP>
 __global__ void __launch_bounds__(128, N == 4 ? 2 : 3)
 k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
@@ -641,44 +641,6 @@ __device__ __forceinline__ int leaf_site(const CfgDesc& c, unsigned eb, int s, i
 }
 
 template <int N>
-__device__ __forceinline__ void fx_leaves(matq<N>& C, long long& retr, const SunSrc<N>& src, const CfgDesc& c, int s, unsigned eb,
-                                          int mu, int nu, fx_guard& g) {
-    fx_zero(C);
-    retr = 0;
-    const int k = c.tw[mu * 4 + nu];
-#pragma unroll 1
-    for (int leaf = 0; leaf < 4; ++leaf) {
-        unsigned w = c_leaf[leaf];
-        matx<N> t;
-        matq<N> q;
-        fx_take_matrix<N>(t, src, w & 1 ? nu : mu, leaf_site(c, eb, s, mu, nu, w & 0xffu), w & 2, g, w & 2 ? -1 : 0);
-        if (k != 0 && leaf_twisted(eb, mu, nu, leaf)) {
-            double zr, zi;
-            centreN<N>(k, zr, zi);
-            fx_scale(t, zr, -zi);
-        }
-#pragma unroll 1
-        for (int m = 1; m < 4; ++m) {
-            w >>= 8;
-            matx<N> b;
-            fx_take_matrix<N>(b, src, w & 1 ? nu : mu, leaf_site(c, eb, s, mu, nu, w & 0xffu), w & 2, g, w & 2 ? -1 : 0);
-            fx_mul_nn<N>(q, t, b);
-            fx_check<N, 27>(q, g);
-            fx_operand_wide<N, 0>(t, q);
-        }
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            if (leaf == 0) retr += q.re[i][i];
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                C.re[i][j] += q.re[i][j];
-                C.im[i][j] += q.im[i][j];
-            }
-        }
-    }
-}
-
-template <int N>
 __device__ __forceinline__ void native_leaves(matN<N>& C, double& retr, const double* __restrict__ base, const CfgDesc& c, int s,
                                               unsigned eb, int mu, int nu) {
     zeroN(C);
@@ -717,6 +679,76 @@ __device__ __forceinline__ void native_leaves(matN<N>& C, double& retr, const do
     }
 }
 
+// The same in fixed point, two leaves at a time: with F, B the staples of U_mu in the plane, L1 + L2^+ goes with
+// U_mu(n) (F - B) and L3 + L4^+ with (F - B) U_mu at n - mu (C - C^+ needs no more), so that a plane takes 10 products
+// instead of 12 and four instead of sixteen links more than once.  Both halves are one loop body: the first
+// is formed transposed.  ah: C - C^+ in units 2^-58, diagonal imaginary parts, then (re, im) above the diagonal; retr: Re
+// Tr[Z* P(n)].  |F| and |F - B| are below 2 and |D| below 4 or the guard is set.  Every thread of the block takes part.
+template <int N>
+__device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& retr, const SunSrc<N>& src, const CfgDesc& c, int s,
+                                          unsigned eb, int mu, int nu, fx_guard& g) {
+    const long long half = fx_round();
+    const int q0 = 2 * ((nu - mu - 1) & 3);
+#pragma unroll
+    for (int r = 0; r < N * N; ++r) ah[r] = 0;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        const int n = h ? bwd(c, eb, s, mu) : s;
+        int xc[4];
+        site_coords(c, n, xc);
+        matq<N> k;
+        fx_zero(k);
+        fx_staples<N, true, false>(k, src, nullptr, 0, c, n, mu, edge_bits(c, xc), g, [&](int back, int, matq<N>& sum) {
+            if (back) return;
+            fx_check<N, 27>(sum, g);
+            if (h == 0) {
+                long long hh = 0, cr = half;
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+                        int rh, rl, ih, il, fh, fl;
+                        const double2 x = src.get(mu, n, i, j, false);
+                        fx_take(x.x, rh, rl, g);
+                        fx_take(x.y, ih, il, g, 0, -1);
+                        fx_split<0>(sum.re[j][i], fh, fl);
+                        fx_mad(hh, cr, rh, rl, fh, fl);
+                        fx_split<0>(sum.im[j][i], fh, fl);
+                        fx_mad(hh, cr, ih, il, fh, fl);
+                    }
+                retr = fx_join(hh, cr);
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    sum.re[i][j] = -sum.re[i][j];
+                    sum.im[i][j] = -sum.im[i][j];
+                }
+        }, q0, q0 + 2);
+        // k = B - F; d = (B - F) U at n - mu, the transpose of U (B - F) at n
+        fx_check<N, 27>(k, g);
+        if (h == 0) fx_transpose(k);
+        matx<N> kx, u;
+        matq<N> d;
+        fx_operand_wide<N, 0>(kx, k);
+        fx_take_matrix<N>(u, src, mu, n, h == 0, g);
+        fx_mul_nn<N>(d, kx, u);
+        fx_check<N, 28>(d, g);
+        int r = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) ah[r++] -= 2 * d.im[i][i];
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = i + 1; j < N; ++j) {
+                const long long re = d.re[i][j] - d.re[j][i];
+                ah[r++] += h ? -re : re;
+                ah[r++] -= d.im[i][j] + d.im[j][i];
+            }
+    }
+}
+
 // Re Tr[A B] for Hermitian A, B
 template <int N>
 __device__ __forceinline__ double retr_prod(const matN<N>& A, const matN<N>& B) {
@@ -736,9 +768,12 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// per-site E, q, p, s summed over each block of kSunSites sites (fixed order)
+// per-site E, q, p, s summed over each block of kSunSites sites (fixed order).  Bound by the integer pipe and latency: SU(2)
+// fits 4 blocks on an SM (two steps and a measurement of 8 x 8x8x16x16 1.49 -> 1.45 ms), SU(3) 3
+// (1.02 -> 0.99 for one step and a measurement of 4 x 6x6x18x18), SU(4) 2 (3 spill: 4.30 -> 4.54 ms on 6x6x24x24).  With the
+// leaves multiplied out one by one, 12 products a plane, these took 1.51, 1.07 and 4.41.
 template <int N, int CAP>
-__global__ void __launch_bounds__(kSunSites, 1)
+__global__ void __launch_bounds__(kSunSites, N == 2 ? 4 : N == 3 ? 3 : 2)
 k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w, double* __restrict__ partial,
               int traceless) {
     __shared__ double red[kSunSites / 32][4];
@@ -746,9 +781,11 @@ k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ 
     if (blk >= B.nblk) return;
     const int ci = find_cfg(B, blk);
     const CfgDesc& c = B.c[ci];
-    const int s = (blk - c.blk0) * kSunSites + threadIdx.x;
+    const int blk_site = (blk - c.blk0) * kSunSites + threadIdx.x;
     double e = 0.0, q = 0.0, p = 0.0, sa = 0.0;
-    if (s < c.V) {
+    {
+        const bool inside = blk_site < c.V;  // the others take part in the barriers
+        const int s = inside ? blk_site : 0;
         int xc[4];
         site_coords(c, s, xc);
         const unsigned eb = edge_bits(c, xc);
@@ -763,17 +800,21 @@ k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ 
             matN<N> G;
             double retr, dev;
             {
-                matq<N> C;
-                long long tr;
-                fx_leaves<N>(C, tr, src, c, s, eb, mu, nu, g);
+                long long ah[N * N], tr;
+                fx_clover<N>(ah, tr, src, c, s, eb, mu, nu, g);
                 retr = (double)tr * 0x1p-58;
                 dev = (double)(((long long)N << kFxBits) - tr) * 0x1p-58;
                 // G = -(i/8)(C - C^+): G_jk = -(i/8)(C_jk - conj(C_kj))
+                int r = 0;
+#pragma unroll
+                for (int i = 0; i < N; ++i) G.e[i][i] = {(double)ah[r++] * 0x1p-61, 0.0};
 #pragma unroll
                 for (int i = 0; i < N; ++i)
 #pragma unroll
-                    for (int j = i; j < N; ++j)
-                        G.e[i][j] = {(double)(C.im[i][j] + C.im[j][i]) * 0x1p-61, -(double)(C.re[i][j] - C.re[j][i]) * 0x1p-61};
+                    for (int j = i + 1; j < N; ++j) {
+                        G.e[i][j] = {(double)ah[r + 1] * 0x1p-61, -(double)ah[r] * 0x1p-61};
+                        r += 2;
+                    }
             }
             if (g.bad()) {
                 matN<N> C;
@@ -800,6 +841,7 @@ k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ 
             sa += dev;
         }
         q *= 1.0 / (4.0 * CUDART_PI * CUDART_PI);
+        if (!inside) e = q = p = sa = 0.0;
     }
     e = warp_sum(e);
     q = warp_sum(q);

@@ -7,11 +7,15 @@
 // entries is three IMAD.WIDE (hi hi; hi lo and lo hi, summed apart; lo lo is below the last bit kept):
 // 13 cycles instead of 64.
 //
-// Accuracy.  Sums are exact: rounding enters once per entry and product, when the sum of the cross
-// terms is rounded to a multiple of 2^-55 (error at most 2^-56 = 1.4e-17), and once when an
-// operand is taken in (below 2^-57).  In FP64 the same entry, a sum of 2N products of size up to 1,
-// carries up to 2N roundings of 2^-54.  So a staple formed here is nearer to its exact value
-// than one formed in FP64.
+// Accuracy.  Operands of 2^-5 and more are exact, smaller ones are cut towards 0 at 2^-58.  Sums are exact: rounding
+// enters once per entry and product, when the sum of the cross terms is rounded to 2^-58 (half a unit at most) and
+// the 2N products lo lo, each below a unit, are replaced by their mean (0.3 of a unit left each, rms).  In FP64 the same
+// entry, a sum of 2N products of size up to 1, carries up to 2N roundings of 2^-54: where the entries are not
+// all small, a staple formed here is nearer to its exact value than one formed in FP64.
+// No rounding leans to one side, as the observables add millions of sites: with operands and sums cut
+// downwards, the lo lo products dropped and cross sums rounded to 2^-55, which costs the same time (a fourth
+// fewer instructions, but on the multiply pipe), S and Q of 4x4x12x12 at amplitude 0.15 were off by 1.5 x 2^-53 S and
+// 0.5 x 2^-53 on the average of 16 fields; now 0.2 and 0.0.
 //
 // Range.  Nothing wraps as long as operand entries stay within the bounds noted at each split: with
 // 2N <= 8 terms of a link and another operand, hi hi sums stay below 8 x 2^30 x 2^29.01 and cross sums
@@ -52,9 +56,9 @@ struct fx_guard {
     __device__ __forceinline__ bool bad() const { return ((top >> 31) | top2) != 0; }
 };
 
-// x -> floor(x 2^58) (negative x: to within one unit, as the bitwise complement of |x|'s image) split
-// into hi, lo.  The mantissa with its leading bit is aligned at the top of 64 bits and
-// shifted right by 1025 - exponent, which leaves x 2^61; shifts past 63 bits give 0.
+// x 2^58, cut towards 0, split into hi, lo.  The mantissa with its leading bit is aligned at the top of 64 bits and
+// shifted right by 1025 - exponent, which leaves |x| 2^61; shifts past 63 bits give 0.  A negative x takes the
+// complement, floor(-|x| 2^58) - 1 once it is cut, and that unit back on lo (1 <= lo <= 2^29 then).
 // `up` takes x 2^up instead (a matrix of small entries keeps its relative precision), flip = -1 takes -x.
 __device__ __forceinline__ void fx_take(double x, int& hi, int& lo, fx_guard& g, unsigned up = 0, int flip = 0) {
     const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
@@ -65,12 +69,14 @@ __device__ __forceinline__ void fx_take(double x, int& hi, int& lo, fx_guard& g,
     asm("shr.b64 %0, %0, %1;" : "+l"(m) : "r"(s));
     const int sg = ((int)h >> 31) ^ flip;
     asm("xor.b32 %0, %1, %2;" : "=r"(hi) : "r"((int)(m >> 32)), "r"(sg));
-    asm("shr.u32 %0, %1, 3;" : "=r"(lo) : "r"((unsigned)m ^ (unsigned)sg));
+    asm("{.reg .u32 t; shr.u32 t, %1, 3; sub.s32 %0, t, %2;}" : "=r"(lo) : "r"((unsigned)m ^ (unsigned)sg), "r"(sg));
 }
 
-// a sum (units 2^-58) -> operand in units 2^(SH-58); |v| < 2 (SH = 0), 4 (SH = 1) or 8 (SH = 2)
-template <int SH>
+// a sum (units 2^-58) -> operand in units 2^(SH-58); |v| < 2 (SH = 0), 4 (SH = 1) or 8 (SH = 2).  ROUND: to the nearest
+// (ties to even, half the values of SH = 1 are ties) for sums that reach an observable, cut downwards otherwise
+template <int SH, bool ROUND = false>
 __device__ __forceinline__ void fx_split(long long v, int& hi, int& lo) {
+    if (ROUND && SH > 0) v += ((1 << SH) / 2 - 1) + (int)(((unsigned)v >> SH) & 1u);
     asm("{.reg .b64 t; shr.s64 t, %1, %2; cvt.u32.u64 %0, t;}" : "=r"(hi) : "l"(v), "n"(29 + SH));
     asm("and.b32 %0, %1, 0x1fffffff;" : "=r"(lo) : "r"((int)(v >> SH)));
 }
@@ -84,14 +90,14 @@ __device__ __forceinline__ void fx_zero(matq<N>& a) {
 }
 
 // a wider operand; its bound (2^(SH+1)) must have been checked
-template <int N, int SH>
+template <int N, int SH, bool ROUND = false>
 __device__ __forceinline__ void fx_operand_wide(matx<N>& o, const matq<N>& v) {
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            fx_split<SH>(v.re[i][j], o.rh[i][j], o.rl[i][j]);
-            fx_split<SH>(v.im[i][j], o.ih[i][j], o.il[i][j]);
+            fx_split<SH, ROUND>(v.re[i][j], o.rh[i][j], o.rl[i][j]);
+            fx_split<SH, ROUND>(v.im[i][j], o.ih[i][j], o.il[i][j]);
         }
 }
 // |entries| < 2^(B - 26), else the guard's second word (the top word of a sum counts in 2^-26)
@@ -116,15 +122,17 @@ __device__ __forceinline__ void fx_mad(long long& hh, long long& cr, int ah, int
     cr = mad_wide(ah, bl, cr);
     cr = mad_wide(al, bh, cr);
 }
-// start of a cross sum: its top word is then the rounded one (opaque: an accumulator of the first
-// multiply-add, not an addition of its own)
+// start of a cross sum (opaque: an accumulator of the first multiply-add, not an addition of its own): half a unit of
+// the hi hi sum, for the rounding, and a quarter of one, the mean of lo lo, for each of TERMS products that add up
+// with one sign (those of both signs cancel)
+template <int TERMS = 0>
 __device__ __forceinline__ long long fx_round() {
     long long r;
-    asm("mov.b64 %0, 0x80000000;" : "=l"(r));
+    asm("mov.b64 %0, %1;" : "=l"(r) : "n"((1ll << 28) + ((long long)TERMS << 27)));
     return r;
 }
-// hi hi sum + rounded cross sum: the cross unit is 2^-29 of the hi hi unit, its top word 8 of them
-__device__ __forceinline__ long long fx_join(long long hh, long long cr) { return mad_wide((int)(cr >> 32), 8, hh); }
+// hi hi sum + rounded cross sum: the cross unit is 2^-29 of the hi hi unit
+__device__ __forceinline__ long long fx_join(long long hh, long long cr) { return hh + (cr >> 29); }
 
 // Re and Im of c + sum_k a_k w_k, w = b or (CONJ) its complex conjugate; minus signs go to a negated copy of a
 // (lo < 2^29, so -lo is exact).
@@ -133,9 +141,8 @@ struct vecx {
     int rh[N], rl[N], ih[N], il[N];
 };
 template <int N, bool CONJ>
-__device__ __forceinline__ void fx_dot(long long& re, long long& im, const vecx<N>& a, const vecx<N>& na, const vecx<N>& b,
-                                       long long half) {
-    long long rc = half, ic = half;
+__device__ __forceinline__ void fx_dot(long long& re, long long& im, const vecx<N>& a, const vecx<N>& na, const vecx<N>& b) {
+    long long rc = fx_round<CONJ ? 2 * N : 0>(), ic = fx_round<CONJ ? 0 : 2 * N>();
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         fx_mad(re, rc, a.rh[k], a.rl[k], b.rh[k], b.rl[k]);
@@ -192,14 +199,13 @@ __device__ __forceinline__ vecx<N> fx_col(const matx<N>& m, int j) {
 // c = a b
 template <int N>
 __device__ __forceinline__ void fx_mul_nn(matq<N>& c, const matx<N>& a, const matx<N>& b) {
-    const long long half = fx_round();
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const vecx<N> r = fx_row(a, i), nr = fx_negated(r);
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             c.re[i][j] = c.im[i][j] = 0;
-            fx_dot<N, false>(c.re[i][j], c.im[i][j], r, nr, fx_col(b, j), half);
+            fx_dot<N, false>(c.re[i][j], c.im[i][j], r, nr, fx_col(b, j));
         }
     }
 }
@@ -208,7 +214,6 @@ __device__ __forceinline__ void fx_mul_nn(matq<N>& c, const matx<N>& a, const ma
 template <int N>
 __device__ __forceinline__ void fx_scale(matx<N>& m, double zr, double zi) {
     fx_guard g;
-    const long long half = fx_round();
     int zrh, zrl, zih, zil;
     fx_take(zr, zrh, zrl, g);
     fx_take(zi, zih, zil, g);
@@ -216,7 +221,7 @@ __device__ __forceinline__ void fx_scale(matx<N>& m, double zr, double zi) {
     for (int i = 0; i < N; ++i)
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            long long rh = 0, ih = 0, rc = half, ic = half;
+            long long rh = 0, ih = 0, rc = fx_round(), ic = fx_round<2>();
             fx_mad(rh, rc, m.rh[i][j], m.rl[i][j], zrh, zrl);
             fx_mad(rh, rc, fx_neg(m.ih[i][j]), fx_neg(m.il[i][j]), zih, zil);
             fx_mad(ih, ic, m.rh[i][j], m.rl[i][j], zih, zil);
@@ -317,7 +322,6 @@ __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shar
                                            int mu, unsigned eb, fx_guard& g, VISIT&& visit, int q0 = 0, int q1 = 6) {
     const int s_mp = fwd(c, eb, s, mu);
     const bool at_mu0 = (eb >> mu) & 1u;  // x_mu = 0: the twisted plaquettes' corner row
-    const long long half = fx_round();
 #pragma unroll 1
     for (int q = q0; q < q1; ++q) {
         const bool back = q & 1;
@@ -363,14 +367,14 @@ __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shar
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 long long re = 0, im = 0;
-                fx_dot<N, true>(re, im, v, nv, fx_row(b, j), half);
+                fx_dot<N, true>(re, im, v, nv, fx_row(b, j));
                 fx_split<0>(re, t.rh[j], t.rl[j]);
                 fx_split<0>(im, t.ih[j], t.il[j]);
                 g.top |= (unsigned)(t.rh[j] + (1 << 30)) | (unsigned)(t.ih[j] + (1 << 30));
             }
             nv = fx_negated(t);
 #pragma unroll
-            for (int j = 0; j < N; ++j) fx_dot<N, true>(sig.re[i][j], sig.im[i][j], t, nv, fx_row(d, j), half);
+            for (int j = 0; j < N; ++j) fx_dot<N, true>(sig.re[i][j], sig.im[i][j], t, nv, fx_row(d, j));
         }
         if (back) fx_transpose(sig);
         fx_check<N, 29>(sig, g);

@@ -194,14 +194,13 @@ __device__ __forceinline__ void take_rotation(rot_fx& o, const rot2& R) {
 // operands, finished rows stay as sums
 template <bool KEEP_I, bool KEEP_J>
 __device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j, const rot_fx& R) {
-    const long long half = fx_round();
 #pragma unroll
     for (int col = 0; col < 3; ++col) {
         vecx<2> p;
         p.rh[0] = u.rh[i][col]; p.rl[0] = u.rl[i][col]; p.ih[0] = u.ih[i][col]; p.il[0] = u.il[i][col];
         p.rh[1] = u.rh[j][col]; p.rl[1] = u.rl[j][col]; p.ih[1] = u.ih[j][col]; p.il[1] = u.il[j][col];
         long long re = 0, im = 0;
-        fx_dot<2, false>(re, im, R.i, R.ni, p, half);
+        fx_dot<2, false>(re, im, R.i, R.ni, p);
         if (KEEP_I) {
             fx_split<0>(re, u.rh[i][col], u.rl[i][col]);
             fx_split<0>(im, u.ih[i][col], u.il[i][col]);
@@ -210,7 +209,7 @@ __device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j
             out.im[i][col] = im;
         }
         re = im = 0;
-        fx_dot<2, false>(re, im, R.j, R.nj, p, half);
+        fx_dot<2, false>(re, im, R.j, R.nj, p);
         if (KEEP_J) {
             fx_split<0>(re, u.rh[j][col], u.rl[j][col]);
             fx_split<0>(im, u.ih[j][col], u.il[j][col]);
@@ -227,7 +226,6 @@ __device__ __forceinline__ void fx_rotate(matq<3>& out, matx<3>& u, int i, int j
 constexpr int kWideW = 25 << 22;  // 6.25 in the top word of a sum in units 2^-56
 template <bool I, bool J>
 __device__ __forceinline__ void fx_rotate_entry(matq<3>& w, int i, int j, int col, const rot_fx& R) {
-    const long long half = fx_round();
     vecx<2> p;
     fx_split<0>(w.re[i][col], p.rh[0], p.rl[0]);
     fx_split<0>(w.im[i][col], p.ih[0], p.il[0]);
@@ -235,11 +233,11 @@ __device__ __forceinline__ void fx_rotate_entry(matq<3>& w, int i, int j, int co
     fx_split<0>(w.im[j][col], p.ih[1], p.il[1]);
     if (I) {
         w.re[i][col] = w.im[i][col] = 0;
-        fx_dot<2, false>(w.re[i][col], w.im[i][col], R.i, R.ni, p, half);
+        fx_dot<2, false>(w.re[i][col], w.im[i][col], R.i, R.ni, p);
     }
     if (J) {
         w.re[j][col] = w.im[j][col] = 0;
-        fx_dot<2, false>(w.re[j][col], w.im[j][col], R.j, R.nj, p, half);
+        fx_dot<2, false>(w.re[j][col], w.im[j][col], R.j, R.nj, p);
     }
 }
 

@@ -178,17 +178,16 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 }
                 const int pl = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
                 fx_shared_link<3>(u, sm.links, mu, lane);
-                const long long half = fx_round();
                 if (!back) {
                     // 3 - Re Tr(U F), the deviation of the twisted plaquette from the unit matrix
-                    long long hh = 0, cr = half;
+                    long long hh = 0, cr = fx_round();
 #pragma unroll
                     for (int i = 0; i < 3; ++i)
 #pragma unroll
                         for (int j = 0; j < 3; ++j) {
                             int rh, rl, ih, il;
-                            fx_split<1>(sum.re[j][i] - kk.re[j][i], rh, rl);
-                            fx_split<1>(sum.im[j][i] - kk.im[j][i], ih, il);
+                            fx_split<1, true>(sum.re[j][i] - kk.re[j][i], rh, rl);
+                            fx_split<1, true>(sum.im[j][i] - kk.im[j][i], ih, il);
                             fx_mad(hh, cr, u.rh[i][j], u.rl[i][j], rh, rl);
                             fx_mad(hh, cr, fx_neg(u.ih[i][j]), fx_neg(u.il[i][j]), ih, il);
                             kk.re[j][i] = 2 * sum.re[j][i] - kk.re[j][i];
@@ -209,7 +208,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 fx_check<3, 28>(kk, g);
                 matx<3> kx;
                 matq<3> t;
-                fx_operand_wide<3, 1>(kx, kk);
+                fx_operand_wide<3, 1, true>(kx, kk);
                 const double unit = nu > mu ? 0x1p-57 : -0x1p-57;
                 fx_mul_nn<3>(t, u, kx);
                 fx_store_ah(cb + (size_t)(pl * 2 + 0) * 9 * Vp, Vp, s, t, unit);

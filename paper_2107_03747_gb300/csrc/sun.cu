@@ -433,7 +433,7 @@ __device__ __forceinline__ unsigned fx_exp_m1<4>(matx<4>& o, const matN<4>& X, f
                 fx_mad(im, ic, y.ih[i][j], y.il[i][j], c1h, c1l);
                 re = fx_join(re, rc);
                 im = fx_join(im, ic);
-                if (!top) fx_dot<N, false>(re, im, r, nr, fx_col(t, j), half);
+                if (!top) fx_dot<N, false>(re, im, r, nr, fx_col(t, j));
                 h.re[i][j] = re;
                 h.im[i][j] = im;
             }
@@ -687,7 +687,6 @@ __device__ __forceinline__ void native_leaves(matN<N>& C, double& retr, const do
 template <int N>
 __device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& retr, const SunSrc<N>& src, const CfgDesc& c, int s,
                                           unsigned eb, int mu, int nu, fx_guard& g) {
-    const long long half = fx_round();
     const int q0 = 2 * ((nu - mu - 1) & 3);
 #pragma unroll
     for (int r = 0; r < N * N; ++r) ah[r] = 0;
@@ -702,7 +701,7 @@ __device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& ret
             if (back) return;
             fx_check<N, 27>(sum, g);
             if (h == 0) {
-                long long hh = 0, cr = half;
+                long long hh = 0, cr = fx_round<2 * N * N>();
 #pragma unroll
                 for (int i = 0; i < N; ++i)
 #pragma unroll

@@ -21,9 +21,10 @@
 // 2N <= 8 terms of a link and another operand, hi hi sums stay below 8 x 2^30 x 2^29.01 and cross sums
 // below 8 (2^30 2^29 + 2^29.01 2^29), both under 2^63.  The
 // fields are arbitrary user data, so every operand is checked as it is taken in: a link entry
-// above 1 + 2^-10 in magnitude (also infinities and NaN), a product T above 2, a staple sum above 8
-// set bits in a guard word; a thread that finds them set repeats its link in FP64 arithmetic, which
-// takes any input.  SU(N) fields never do.
+// above 1 + 2^-10 in magnitude (also infinities and NaN), a product T above 2, a staple sum above 8, an entry of Omega
+// above 32 (the trace adds up to four) set bits in a guard word; a thread that finds them set repeats its link in FP64
+// arithmetic, which takes any input.  SU(N) fields never do.  Sums are tested in 64 bits, before a split narrows them:
+// entries of size 1 that add up in phase make T as large as 2N sqrt 2, which the 32 bits of hi fold back.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -343,6 +344,7 @@ __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shar
         }
         if (SHARE && !back) fx_shared_link<N>(d, *sh, nu, lane);
         else fx_take_matrix<N>(d, src, nu, sc, back, g);
+        unsigned wide = 0;  // top words of T, in 2^-26, plus 2: 28 bits while |T| < 2
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             vecx<N> v, t;
@@ -368,15 +370,16 @@ __device__ __forceinline__ void fx_staples(matq<N>& sig, SRC& src, const fx_shar
             for (int j = 0; j < N; ++j) {
                 long long re = 0, im = 0;
                 fx_dot<N, true>(re, im, v, nv, fx_row(b, j));
+                wide |= (unsigned)((int)(re >> 32) + (1 << 27)) | (unsigned)((int)(im >> 32) + (1 << 27));
                 fx_split<0>(re, t.rh[j], t.rl[j]);
                 fx_split<0>(im, t.ih[j], t.il[j]);
-                g.top |= (unsigned)(t.rh[j] + (1 << 30)) | (unsigned)(t.ih[j] + (1 << 30));
             }
             nv = fx_negated(t);
 #pragma unroll
             for (int j = 0; j < N; ++j) fx_dot<N, true>(sig.re[i][j], sig.im[i][j], t, nv, fx_row(d, j));
         }
         if (back) fx_transpose(sig);
+        g.top2 |= wide >> 28;
         fx_check<N, 29>(sig, g);
         visit(q & 1, nu, sig);
     }

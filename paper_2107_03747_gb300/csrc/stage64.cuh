@@ -179,21 +179,38 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 const int pl = c_plane_of[mu < nu ? mu : nu][mu < nu ? nu : mu];
                 fx_shared_link<3>(u, sm.links, mu, lane);
                 if (!back) {
-                    // 3 - Re Tr(U F), the deviation of the twisted plaquette from the unit matrix
-                    long long hh = 0, cr = fx_round();
+                    // 3 - Re Tr(U F), the deviation of the twisted plaquette from the unit matrix.  With entries of F below
+                    // 2, the 18 hi hi products stay below 2^62.2 and the cross sum of a row below 2^61.6.
 #pragma unroll
                     for (int i = 0; i < 3; ++i)
 #pragma unroll
                         for (int j = 0; j < 3; ++j) {
+                            kk.re[i][j] = sum.re[i][j] - kk.re[i][j];
+                            kk.im[i][j] = sum.im[i][j] - kk.im[i][j];
+                        }
+                    fx_check<3, 27>(kk, g);
+                    long long hh = 0;
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        long long cr = fx_round();
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) {
                             int rh, rl, ih, il;
-                            fx_split<1, true>(sum.re[j][i] - kk.re[j][i], rh, rl);
-                            fx_split<1, true>(sum.im[j][i] - kk.im[j][i], ih, il);
+                            fx_split<1, true>(kk.re[j][i], rh, rl);
+                            fx_split<1, true>(kk.im[j][i], ih, il);
                             fx_mad(hh, cr, u.rh[i][j], u.rl[i][j], rh, rl);
                             fx_mad(hh, cr, fx_neg(u.ih[i][j]), fx_neg(u.il[i][j]), ih, il);
-                            kk.re[j][i] = 2 * sum.re[j][i] - kk.re[j][i];
-                            kk.im[j][i] = 2 * sum.im[j][i] - kk.im[j][i];
                         }
-                    cb[(size_t)(108 + pl) * Vp + s] = (double)((3ll << 57) - fx_join(hh, cr)) * 0x1p-57;
+                        hh = fx_join(hh, cr);
+                    }
+                    cb[(size_t)(108 + pl) * Vp + s] = (double)((3ll << 57) - hh) * 0x1p-57;
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) {
+                            kk.re[i][j] += sum.re[i][j];
+                            kk.im[i][j] += sum.im[i][j];
+                        }
                     return;
                 }
                 // K = F - B; D1 = U K (site n), D2 = K U (site n + mu).  A plane built through its second
@@ -257,6 +274,7 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
             matq<3> om;
             fx_operand_wide<3, 2>(sx, sig);
             fx_mul_nn<3>(om, u, sx);
+            fx_check<3, 29>(om, g);
             const double tr = (double)(om.im[0][0] + om.im[1][1] + om.im[2][2]) * (1.0 / 3.0);
             z.v[0] = 0x1p-56 * (tr - (double)om.im[0][0]);
             z.v[1] = 0x1p-56 * (tr - (double)om.im[1][1]);

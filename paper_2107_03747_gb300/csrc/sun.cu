@@ -529,6 +529,7 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
         fx_operand_wide<N, 2>(sx, sig);
         own_link();
         fx_mul_nn<N>(om, u, sx);
+        fx_check<N, 29>(om, g);
         long long tr = 0;
 #pragma unroll
         for (int i = 0; i < N; ++i) tr += om.im[i][i];
@@ -683,7 +684,10 @@ __device__ __forceinline__ void native_leaves(matN<N>& C, double& retr, const do
 // U_mu(n) (F - B) and L3 + L4^+ with (F - B) U_mu at n - mu (C - C^+ needs no more), so that a plane takes 10 products
 // instead of 12 and four instead of sixteen links more than once.  Both halves are one loop body: the first
 // is formed transposed.  ah: C - C^+ in units 2^-58, diagonal imaginary parts, then (re, im) above the diagonal; retr: Re
-// Tr[Z* P(n)].  |F| and |F - B| are below 2 and |D| below 4 or the guard is set.  Every thread of the block takes part.
+// Tr[Z* P(n)], up to 4 N^2, in units 2^(kTraceShift<N> - 58).  |F| and |F - B| are below 2 and |D| below 4 or the guard is
+// set.  Every thread of the block takes part.
+template <int N>
+constexpr int kTraceShift = N - 2;  // 2 N^2 products of a link and F in these units stay below 2^62.2
 template <int N>
 __device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& retr, const SunSrc<N>& src, const CfgDesc& c, int s,
                                           unsigned eb, int mu, int nu, fx_guard& g) {
@@ -701,21 +705,24 @@ __device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& ret
             if (back) return;
             fx_check<N, 27>(sum, g);
             if (h == 0) {
-                long long hh = 0, cr = fx_round<2 * N * N>();
+                long long hh = 0;
 #pragma unroll
-                for (int i = 0; i < N; ++i)
+                for (int i = 0; i < N; ++i) {
+                    long long cr = fx_round<2 * N>();
 #pragma unroll
                     for (int j = 0; j < N; ++j) {
                         int rh, rl, ih, il, fh, fl;
                         const double2 x = src.get(mu, n, i, j, false);
                         fx_take(x.x, rh, rl, g);
                         fx_take(x.y, ih, il, g, 0, -1);
-                        fx_split<0>(sum.re[j][i], fh, fl);
+                        fx_split<kTraceShift<N>, true>(sum.re[j][i], fh, fl);
                         fx_mad(hh, cr, rh, rl, fh, fl);
-                        fx_split<0>(sum.im[j][i], fh, fl);
+                        fx_split<kTraceShift<N>, true>(sum.im[j][i], fh, fl);
                         fx_mad(hh, cr, ih, il, fh, fl);
                     }
-                retr = fx_join(hh, cr);
+                    hh = fx_join(hh, cr);
+                }
+                retr = hh;
             }
 #pragma unroll
             for (int i = 0; i < N; ++i)
@@ -801,8 +808,9 @@ k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ 
             {
                 long long ah[N * N], tr;
                 fx_clover<N>(ah, tr, src, c, s, eb, mu, nu, g);
-                retr = (double)tr * 0x1p-58;
-                dev = (double)(((long long)N << kFxBits) - tr) * 0x1p-58;
+                constexpr double unit = 0x1p-58 * (1 << kTraceShift<N>);
+                retr = (double)tr * unit;
+                dev = (double)(((long long)N << (kFxBits - kTraceShift<N>)) - tr) * unit;
                 // G = -(i/8)(C - C^+): G_jk = -(i/8)(C_jk - conj(C_kj))
                 int r = 0;
 #pragma unroll

@@ -1,0 +1,98 @@
+"""Fields on which the fixed-point products of the double-precision kernels (csrc/fixed.cuh) must give way to FP64
+arithmetic or widen their sums, against the oracle: links whose entries add up in phase, so that T = V B^+, the
+staples, Omega and the traces come out far beyond those of unitary matrices.
+
+Tolerances.  FP64 arithmetic carries about 6N + 6 roundings of U = 2^-53 along a link: 100 U of the size of the terms
+covers them in the worst case.
+"""
+import numpy as np
+import pytest
+
+from oracle import tgf_oracle as O
+from paper_2107_03747_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+L = (4, 2, 6, 4)  # 192 sites
+TW = I.default_twist(1)
+
+
+def in_phase(kind, N):
+    J = np.ones((N, N))
+    shape = (L[3], L[2], L[1], L[0], 4, N, N)
+    x3, x2, x1, x0 = np.meshgrid(*(np.arange(L[d]) for d in (3, 2, 1, 0)), indexing="ij")
+    x = (x0, x1, x2, x3)
+    u = np.empty(shape, complex)
+    if kind == "all":  # T = 2N
+        u[...] = (1 + 1j) * J
+    elif kind == "nine_tenths":  # T = 1.62 N
+        u[...] = 0.9 * (1 + 1j) * J
+    elif kind == "phases":  # T = 2N times a fourth root of 1
+        ph = 1j ** np.random.default_rng(3).integers(0, 4, shape[:5])
+        u[...] = ph[..., None, None] * (1 + 1j) * J
+    elif kind == "below_six":  # T just inside 6 for N = 3
+        u[...] = 0.9999 * (1 + 1j) * J
+    elif kind == "omega":  # |T| < 2 and staple sums of 7.5 (1 +- i), but Im Tr Omega = 15 N^2
+        a = np.sqrt(7.5 / (6 * N * N))
+        u[..., 0, :, :] = (1 + 1j) * J
+        for nu in (1, 2, 3):
+            ph = np.exp(0.5j * np.pi * x0 * (-1.0) ** x[nu])
+            u[..., nu, :, :] = a * ph[..., None, None] * J
+    elif kind == "trace":  # staples of 1.9 (1 - i) in the planes of direction 0: Re Tr(U F) = 3.8 N^2
+        u[...] = np.sqrt(1.9) / N * J
+        u[..., 0, :, :] = (1 + 1j) * J
+    return u
+
+
+IN_PHASE = ["all", "nine_tenths", "phases", "below_six", "omega", "trace"]
+
+
+def batch(tgf, N, tw=None):
+    if N is None:
+        return tgf.FlowBatch([L], "fp64", tw, any_extents=True)
+    return tgf.SunBatch(N, [L], tw, any_extents=True)
+
+
+@pytest.mark.parametrize("N", [None, 2, 3, 4])  # None: the SU(3) kernels
+@pytest.mark.parametrize("kind", IN_PHASE)
+def test_stage_of_links_in_phase(tgf, kind, N):
+    n = N or 3
+    u = in_phase(kind, n)
+    b = batch(tgf, N)
+    b.set_links([u])
+    h = 0.02 / (6 * n ** 3 * np.abs(u).max() ** 4)  # X stays small whatever the force
+    b.stage(1, h)
+    ref = np.matmul(O.expm(0.25 * h * O.force(u, TW)), u)
+    assert np.abs(b.get_links()[0] - ref).max() <= 100 * U * np.abs(u).max()
+
+
+@pytest.mark.parametrize("N", [None, 2, 3, 4])
+@pytest.mark.parametrize("kind", IN_PHASE)
+def test_measure_of_links_in_phase(tgf, kind, N):
+    n = N or 3
+    u = in_phase(kind, n)
+    b = batch(tgf, N)
+    b.set_links([u])
+    g = b.measure()[0].tolist()
+    o = O.measure(u, TW)
+    V = u[..., 0, 0, 0].size
+    size = n ** 3 * np.abs(u).max() ** 4  # of a leaf's entry
+    assert abs(g[4] - o["S"]) <= 100 * U * 6 * V * n * size
+    assert abs(g[1] - o["E"]) <= 100 * U * 6 * n * n * size ** 2
+    assert abs(g[2] - o["Q"]) <= 100 * U * V * n * n * size ** 2
+
+
+@pytest.mark.parametrize("kind", IN_PHASE)
+def test_measured_flow_step_of_links_in_phase(tgf, kind):
+    """The clover halves of a measured stage are those of the measurement alone."""
+    u = in_phase(kind, 3)
+    b = batch(tgf, None)
+    b.set_links([u])
+    ref = b.measure()[0].tolist()
+    obs, _ = b.flow(1e-6, 1e-6)
+    got = obs.cpu().numpy()[0, 0]
+    size = 27 * np.abs(u).max() ** 4
+    V = u[..., 0, 0, 0].size
+    assert abs(got[4] - ref[4]) <= 100 * U * 6 * V * 3 * size
+    assert abs(got[1] - ref[1]) <= 100 * U * 54 * size ** 2

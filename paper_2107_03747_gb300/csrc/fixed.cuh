@@ -11,7 +11,7 @@
 // enters once per entry and product, when the sum of the cross terms is rounded to 2^-58 (half a unit at most) and
 // the 2N products lo lo, each below a unit, are replaced by their mean (0.3 of a unit left each, rms).  In FP64 the same
 // entry, a sum of 2N products of size up to 1, carries up to 2N roundings of 2^-54: where the entries are not
-// all small, a staple formed here is nearer to its exact value than one formed in FP64.
+// all small (fx_rough), a staple formed here is nearer to its exact value than one formed in FP64.
 // No rounding leans to one side, as the observables add millions of sites: with operands and sums cut
 // downwards, the lo lo products dropped and cross sums rounded to 2^-55, which costs the same time (a fourth
 // fewer instructions, but on the multiply pipe), S and Q of 4x4x12x12 at amplitude 0.15 were off by 1.5 x 2^-53 S and
@@ -54,6 +54,8 @@ constexpr int kFxBits = 58;
 struct fx_guard {
     unsigned top = 0;   // bit 31: an operand outside its bound
     unsigned top2 = 0;  // not 0: a sum outside its bound
+    unsigned far = 0;   // bits 26-28: an entry away from 0 and +-1 (fx_rough)
+    __device__ __forceinline__ bool rough() const { return (far & 0x1c000000u) != 0; }
     __device__ __forceinline__ bool bad() const { return ((top >> 31) | top2) != 0; }
 };
 
@@ -271,8 +273,25 @@ __device__ __forceinline__ void fx_transpose(matq<N>& m) {
         }
 }
 
-// a link, transposed if `tr`; flip = -1 conjugates it
-template <int N, class SRC>
+// Weak fields.  A resolution of 2^-58 for every entry serves fields whose links are of size 1 all over.  Near the unit matrix
+// (or any field of one entry +-1, +-i per row and column) force and clover come from the small entries, which FP64 holds
+// to 53 bits and whose products it rounds relative to their own size.  So a link takes the FP64 path if it is weak: if
+// every real and imaginary part of it and of the 18 links that its staples read is within 2^-4 of 0 or +-1, or if the links that
+// its block shares are.  Error of a link's force relative to its largest entry (rms, SU(3), links exp(i amp omega T);
+// of a clover half a quarter more), and how many are weak by themselves:
+//    amp          0.3      0.1      0.07     0.05     0.03     0.01     1e-4     1e-8
+//    FP64         6.8e-17  6.2e-17  6.2e-17  6.3e-17  6.2e-17  6.4e-17  6.4e-17  6.3e-17
+//    fixed point  2.6e-17  3.1e-17  3.5e-17  4.5e-17  6.8e-17  2e-16    2e-14    2e-10
+//    weak         0        0        0        7 %      98 %     all      all      all
+// A rough field pays up to 1 % for the test of the links that it shares.  A weak one runs at the FP64 pipe's rate: two
+// steps of 4 x 8x8x24x24 take 13.6 ms at amp 1e-6, 14.6 at 0.05 where blocks do both, 4.2 at 0.07, 3.7 above.
+__device__ __forceinline__ bool fx_rough(double2 x) {
+    constexpr unsigned lo = 0x3FB00000u, n = 0x3FEE0000u - lo;  // top words of 2^-4 and 1 - 2^-4
+    return ((unsigned)__double2hiint(x.x) & 0x7fffffffu) - lo < n || ((unsigned)__double2hiint(x.y) & 0x7fffffffu) - lo < n;
+}
+
+// a link, transposed if `tr`; flip = -1 conjugates it; TEST: its entries go to the guard's far
+template <int N, bool TEST = false, class SRC>
 __device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, int site, bool tr, fx_guard& g, int flip = 0) {
     double2 x[N][N];
 #pragma unroll
@@ -285,15 +304,17 @@ __device__ __forceinline__ void fx_take_matrix(matx<N>& o, SRC& src, int dir, in
         for (int j = 0; j < N; ++j) {
             fx_take(x[i][j].x, o.rh[i][j], o.rl[i][j], g);
             fx_take(x[i][j].y, o.ih[i][j], o.il[i][j], g, 0, flip);
+            // hi, in 2^-29, plus 2^25: bits 26-28 are clear within 2^25 of 0 and +-2^29
+            if (TEST) g.far |= (unsigned)(o.rh[i][j] + (1 << 25)) | (unsigned)(o.ih[i][j] + (1 << 25));
         }
 }
 
 // Links that several warps of a block need, taken as operands once and shared: [dir] U_dir(n) and [4 + dir] U_dir(n - dir)
-// of the block's 32 sites, entry by entry (re hi, lo, im hi, lo), and the guard words of what was taken.
+// of the block's 32 sites, entry by entry (re hi, lo, im hi, lo), and whether each is out of range (bit 0) and rough (bit 26).
 template <int N>
 struct fx_shared {
     int4 u[8][N * N][32];
-    unsigned bad[8][32];
+    unsigned flags[8][32];
 };
 template <int N>
 __device__ __forceinline__ void fx_share(fx_shared<N>& sh, int m, int lane, const matx<N>& o, const fx_guard& g) {
@@ -301,7 +322,21 @@ __device__ __forceinline__ void fx_share(fx_shared<N>& sh, int m, int lane, cons
     for (int i = 0; i < N; ++i)
 #pragma unroll
         for (int j = 0; j < N; ++j) sh.u[m][i * N + j][lane] = make_int4(o.rh[i][j], o.rl[i][j], o.ih[i][j], o.il[i][j]);
-    sh.bad[m][lane] = g.bad();
+    sh.flags[m][lane] = (unsigned)g.bad() | (g.rough() ? 1u << 26 : 0u);
+}
+// The flags of the links at lane's site that the link in direction mu reads, into its guard; whether none of the block's links
+// is rough.  All lanes of the warp.
+template <int N>
+__device__ __forceinline__ bool fx_shared_flags(fx_guard& g, const fx_shared<N>& sh, int mu, int lane) {
+    unsigned f = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const unsigned v = sh.flags[m][lane];
+        f |= v;
+        if (m != 4 + mu) g.far |= v;
+    }
+    g.top2 |= f & 1u;
+    return !__any_sync(0xffffffffu, f >> 26);
 }
 template <int N>
 __device__ __forceinline__ void fx_shared_link(matx<N>& o, const fx_shared<N>& sh, int m, int lane) {
@@ -403,6 +438,29 @@ struct Su3Src {
     }
     static __device__ __forceinline__ void centre(int k, double& zr, double& zi) { tgf::centre<double>(k, zr, zi); }
 };
+
+// Whether a link, and all links that the staples of U_mu(s) read, are near 0 and +-1
+template <int N, class SRC>
+__device__ __forceinline__ bool fx_near(const SRC& src, int dir, int s) {
+    bool rough = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int j = 0; j < N; ++j) rough |= fx_rough(src.get(dir, s, i, j, false));
+    return !rough;
+}
+template <int N, class SRC>
+__device__ __forceinline__ bool fx_near_staples(const SRC& src, const CfgDesc& c, unsigned eb, int s, int mu) {
+#pragma unroll 1
+    for (int q = 0; q < 18; ++q) {
+        // U_nu at n, n - nu, n + mu, n + mu - nu, U_mu at n + nu, n - nu
+        const int nu = (mu + 1 + q % 3) & 3, k = q / 3;
+        int t = (k & 1) ? bwd(c, eb, s, nu) : k == 4 ? fwd(c, eb, s, nu) : s;
+        if (k == 2 || k == 3) t = fwd(c, eb, t, mu);  // x_mu(n - nu) = x_mu(n)
+        if (!fx_near<N>(src, k < 4 ? nu : mu, t)) return false;
+    }
+    return true;
+}
 
 // The largest up <= 40 for which every entry of m, times 2^up, stays below 1 in magnitude.
 template <int N>

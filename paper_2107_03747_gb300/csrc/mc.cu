@@ -89,7 +89,9 @@ __device__ bool sample_x0(double alpha, uint64_t key, uint64_t c0, double& x0) {
     return false;
 }
 
-// Omega = U_mu(n) Sigma_mu(n) in FP64, for links whose staples leave the range of fixed.cuh
+// Omega = U_mu(n) Sigma_mu(n) in FP64, for links whose staples leave the range of fixed.cuh.  Weak links (fx_rough) stay in
+// fixed point here: every call begins with a heat-bath pass, whose sqrt(1 - x0^2) has a relative error of 2^-53 / amp^2
+// in FP64 on links of amplitude amp, more than the fixed-point staples' 2^-58 / amp at any amp.
 __device__ __forceinline__ void native_omega(mat3<double>& om, const double* __restrict__ base, int Vp, const CfgDesc& c, int s,
                                              unsigned eb, int mu) {
     auto link = [&](int dir, int site, mat3<double>& u) { Store<P64>::load(base + (size_t)dir * 18 * Vp, Vp, site, u); };

@@ -46,10 +46,12 @@ __device__ __forceinline__ void rk3_x(alg8<double>& x, const alg8<double>& z, do
 }
 
 // The force (and the clover halves) in FP64 throughout, for links whose fields leave the range of
-// fixed.cuh (entries above 1 + 2^-10, infinities, NaN): any input, at the FP64 pipe's rate.
+// fixed.cuh (entries above 1 + 2^-10, infinities, NaN) and for weak ones (fx_rough): any input, at the FP64 pipe's rate.
+// trace: also the plaquette deviations 3 - Re Tr(U F), which fixed point has to 2^-57 where it is in range.
 template <int MODE>
 __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c, const double* __restrict__ base,
-                                               double* __restrict__ cb, int s, int mu, unsigned eb, int dn0 = 1, int dn1 = 4) {
+                                               double* __restrict__ cb, int s, int mu, unsigned eb, bool trace, int dn0 = 1,
+                                               int dn1 = 4) {
     const int Vp = c.Vp;
     auto link = [&](int dir, int site, mat3<double>& u) { Store<P64>::load(base + (size_t)dir * 18 * Vp, Vp, site, u); };
     mat3<double> sig, a, b, t, f;
@@ -88,7 +90,7 @@ __device__ __forceinline__ void native_force64(alg8<double>& z, const CfgDesc& c
 #pragma unroll
                 for (int j = 0; j < 3; ++j)
                     rt = fma(a.e[i][j].re, f.e[j][i].re, fma(-a.e[i][j].im, f.e[j][i].im, rt));
-            cb[(size_t)(108 + pl) * Vp + s] = 3.0 - rt;
+            if (trace) cb[(size_t)(108 + pl) * Vp + s] = 3.0 - rt;
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -152,14 +154,19 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
         fx_zero(sig);
         if (MODE != 0) fx_zero(kk);
         __syncthreads();  // the block before is done with the shared memory
+        bool rough = false;
 #pragma unroll 1
         for (int m = warp; m < 8; m += (int)blockDim.x >> 5) {
             fx_guard gl;
-            fx_take_matrix<3>(u, src, m & 3, m < 4 ? s : bwd(c, eb, s, m & 3), false, gl);
+            fx_take_matrix<3, true>(u, src, m & 3, m < 4 ? s : bwd(c, eb, s, m & 3), false, gl);
             fx_share<3>(sm.links, m, lane, u, gl);
+            rough |= gl.rough();
         }
+        // a block of weak links needs no fixed-point staples (but for the plaquette deviations of a measured stage)
+        const bool skip = MODE == 0 && !__syncthreads_or(rough);
+        auto weak = [&]() { return !g.rough() && fx_near_staples<3>(src, c, eb, s, mu); };
 #pragma unroll 1
-        for (int it = 0; it < (MODE == 2 && !WIDE ? 2 : 1); ++it) {
+        for (int it = skip ? 1 : 0; it < (MODE == 2 && !WIDE ? 2 : 1); ++it) {
             int q0 = WIDE ? 2 * part : 0, q1 = WIDE ? 2 * part + 2 : 6;
             if (MODE == 2) {
                 const int e = WIDE ? warp : 2 * warp + it;
@@ -233,14 +240,15 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
                 fx_store_ah(cb + (size_t)(pl * 2 + 1) * 9 * Vp, Vp, fwd(c, eb, s, mu), t, unit);
                 kk = sum;
             }, q0, q1);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) g.top2 |= sm.links.bad[m][lane];
-            if (MODE == 2 && valid && g.bad()) {
+            if (MODE == 2) {
+                const bool all_near = fx_shared_flags<3>(g, sm.links, mu, lane);
                 alg8<double> z;
-                native_force64<MODE>(z, c, base, cb, s, mu, eb, q0 / 2 + 1, q0 / 2 + 2);
+                if (valid && (g.bad() || all_near || weak()))
+                    native_force64<MODE>(z, c, base, cb, s, mu, eb, g.bad(), q0 / 2 + 1, q0 / 2 + 2);
             }
         }
         if (MODE == 2) continue;
+        const bool all_near = fx_shared_flags<3>(g, sm.links, mu, lane);
         fx_shared_link<3>(u, sm.links, mu, lane);
         if constexpr (WIDE && MODE != 2) {
             const int lt = threadIdx.x & 127;
@@ -285,7 +293,10 @@ k_stage64(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in
             z.v[6] = 0x1p-57 * (double)(om.re[2][1] - om.re[1][2]);
             z.v[7] = -0x1p-57 * (double)(om.im[1][2] + om.im[2][1]);
         }
-        if (g.bad()) native_force64<MODE>(z, c, base, cb, s, mu, eb);
+        if (g.bad() || all_near || weak()) {
+            native_force64<MODE>(z, c, base, cb, s, mu, eb, g.bad());
+            g.top2 = 1;
+        }
         rk3_x<STAGE>(x, z, c.h, xb, Vp, s);
         mat3<double> e, w;
         matx<3> ex;

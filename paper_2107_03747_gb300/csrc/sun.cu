@@ -278,7 +278,7 @@ struct SunSrc {
     static __device__ __forceinline__ void centre(int k, double& zr, double& zi) { centreN<N>(k, zr, zi); }
 };
 
-// Omega = U Sigma in FP64, for links whose staples leave the range of fixed.cuh
+// Omega = U Sigma in FP64, for links whose staples leave the range of fixed.cuh and for weak ones (fx_rough)
 template <int N>
 __device__ __forceinline__ void native_omegaN(matN<N>& om, const CfgDesc& c, const double* __restrict__ base, int s, int mu,
                                               unsigned eb) {
@@ -502,28 +502,28 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
     extern __shared__ __align__(16) unsigned char s_links[];
     fx_shared<N>& links = *reinterpret_cast<fx_shared<N>*>(s_links);
     matx<N> u;
+    bool all_near = false;
     if (SHARE) {
+        bool rough = false;
 #pragma unroll 1
         for (int m = mu; m < 8; m += 4) {
             fx_guard gl;
-            fx_take_matrix<N>(u, src, mu, m < 4 ? s : bwd(c, eb, s, mu), false, gl);
+            fx_take_matrix<N, true>(u, src, mu, m < 4 ? s : bwd(c, eb, s, mu), false, gl);
             fx_share<N>(links, m, lane, u, gl);
+            rough |= gl.rough();
         }
+        all_near = !__syncthreads_or(rough);  // a block of weak links needs no fixed-point staples
     }
     auto own_link = [&]() {
         if (SHARE) fx_shared_link<N>(u, links, mu, lane);
-        else fx_take_matrix<N>(u, src, mu, s, false, g);
+        else fx_take_matrix<N, true>(u, src, mu, s, false, g);
     };
     matN<N> X;
     double x[N * N];  // Z, then X: diagonal imaginary parts, then (re, im) above the diagonal
-    {
+    if (!all_near) {
         matq<N> sig, om;
         fx_zero(sig);
         fx_staples<N, true, SHARE>(sig, src, &links, lane, c, s, mu, eb, g, [](int, int, const matq<N>&) {});
-        if (!valid) return;
-        if (SHARE)
-#pragma unroll
-            for (int m = 0; m < 8; ++m) g.top2 |= links.bad[m][lane];
         // Omega = U Sigma (units 2^-56); Z = -P_ta(Omega) = -(Omega - Omega^+)/2 + tr(Omega - Omega^+)/(2N)
         matx<N> sx;
         fx_operand_wide<N, 2>(sx, sig);
@@ -545,7 +545,10 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
                 x[r++] = -0x1p-57 * (double)(om.im[i][j] + om.im[j][i]);
             }
     }
-    if (g.bad()) {
+    if (SHARE) fx_shared_flags<N>(g, links, mu, lane);
+    if (!valid) return;
+    if (g.bad() || all_near || (!g.rough() && fx_near_staples<N>(src, c, eb, s, mu))) {
+        g.top2 = 1;
         matN<N> t;
         native_omegaN<N>(t, c, base, s, mu, eb);
         double trim = 0.0;
@@ -586,7 +589,8 @@ k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_
             r += 2;
         }
     matx<N> ex;
-    const unsigned up = fx_exp_m1<N>(ex, X, g);
+    // (left out where FP64 follows only for SU(4): its six products; the branch costs SU(3) 7 % and SU(2) 3 %)
+    const unsigned up = N == 4 && g.bad() ? 0u : fx_exp_m1<N>(ex, X, g);
     matN<N> w;
     loadN<N>(base, Vp, mu, s, w);
     if (g.bad()) {
@@ -738,7 +742,7 @@ __device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& ret
         matx<N> kx, u;
         matq<N> d;
         fx_operand_wide<N, 0>(kx, k);
-        fx_take_matrix<N>(u, src, mu, n, h == 0, g);
+        fx_take_matrix<N, true>(u, src, mu, n, h == 0, g);
         fx_mul_nn<N>(d, kx, u);
         fx_check<N, 28>(d, g);
         int r = 0;
@@ -753,6 +757,21 @@ __device__ __forceinline__ void fx_clover(long long (&ah)[N * N], long long& ret
                 ah[r++] -= d.im[i][j] + d.im[j][i];
             }
     }
+}
+
+// Whether the 12 links of a plane's leaves are near 0 and +-1 (fx_rough): its clover is formed in FP64 then (Re Tr[Z* P],
+// of the size of N, stays as it is).
+template <int N>
+__device__ __forceinline__ bool weak_plane(const SunSrc<N>& src, const CfgDesc& c, unsigned eb, int s, int mu, int nu) {
+#pragma unroll 1
+    for (int q = 0; q < 12; ++q) {
+        // direction a at n and n - a, each at 0, + and - one step of the other one
+        const int a = q & 1 ? nu : mu, b = q & 1 ? mu : nu, k = q >> 2;
+        int t = k == 1 ? fwd(c, eb, s, b) : k == 2 ? bwd(c, eb, s, b) : s;
+        if (q & 2) t = bwd(c, eb, t, a);
+        if (!fx_near<N>(src, a, t)) return false;
+    }
+    return true;
 }
 
 // Re Tr[A B] for Hermitian A, B
@@ -823,10 +842,14 @@ k_sun_measure(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ 
                         r += 2;
                     }
             }
-            if (g.bad()) {
+            if (g.bad() || (!g.rough() && weak_plane<N>(src, c, eb, s, mu, nu))) {
                 matN<N> C;
-                native_leaves<N>(C, retr, base, c, s, eb, mu, nu);
-                dev = N - retr;
+                double rt;
+                native_leaves<N>(C, rt, base, c, s, eb, mu, nu);
+                if (g.bad()) {
+                    retr = rt;
+                    dev = N - rt;
+                }
 #pragma unroll
                 for (int i = 0; i < N; ++i)
 #pragma unroll

@@ -282,9 +282,9 @@ __device__ __forceinline__ void fx_transpose(matq<N>& m) {
 //    amp          0.3      0.1      0.07     0.05     0.03     0.01     1e-4     1e-8
 //    FP64         6.8e-17  6.2e-17  6.2e-17  6.3e-17  6.2e-17  6.4e-17  6.4e-17  6.3e-17
 //    fixed point  2.6e-17  3.1e-17  3.5e-17  4.5e-17  6.8e-17  2e-16    2e-14    2e-10
-//    weak         0        0        0        7 %      98 %     all      all      all
+//    weak         0        0        0        4 %      98 %     all      all      all
 // A rough field pays up to 1 % for the test of the links that it shares.  A weak one runs at the FP64 pipe's rate: two
-// steps of 4 x 8x8x24x24 take 13.6 ms at amp 1e-6, 14.6 at 0.05 where blocks do both, 4.2 at 0.07, 3.7 above.
+// steps of 4 x 8x8x24x24 take 13.6 ms at amp 1e-6, 14.6 at 0.05 where most warps do both, 4.2 at 0.07, 3.7 above.
 __device__ __forceinline__ bool fx_rough(double2 x) {
     constexpr unsigned lo = 0x3FB00000u, n = 0x3FEE0000u - lo;  // top words of 2^-4 and 1 - 2^-4
     return ((unsigned)__double2hiint(x.x) & 0x7fffffffu) - lo < n || ((unsigned)__double2hiint(x.y) & 0x7fffffffu) - lo < n;

@@ -369,8 +369,8 @@ __constant__ long long c_inv_fact[12] = {1ll << 58, 1ll << 58, (1ll << 58) / 2, 
 
 // SU(4): the Taylor polynomial of expN (same degrees), in fixed point: Y and Y' = 2^up Y as operands, M = Y^2,
 // T = B_1 + M (B_2 + ...) with B_j = 1/(2j)! + Y/(2j+1)!, then exp(Y) - 1 = Y + M T and, s times,
-// exp(2Y) - 1 = 2 (exp(Y) - 1) + (exp(Y) - 1)^2.  M and the last product carry the factor 2^up, so that
-// the small matrix keeps its relative precision.
+// exp(2Y) - 1 = 2 (exp(Y) - 1) + (exp(Y) - 1)^2.  M, the last product and the Y that is added to it carry the factor
+// 2^up, so that the small matrix keeps its relative precision.
 template <>
 __device__ __forceinline__ unsigned fx_exp_m1<4>(matx<4>& o, const matN<4>& X, fx_guard& g) {
     constexpr int N = 4;
@@ -444,12 +444,18 @@ __device__ __forceinline__ unsigned fx_exp_m1<4>(matx<4>& o, const matN<4>& X, f
     matx<N> mu_;
     fx_operand_wide<N, 0>(mu_, q);
     fx_mul_nn<N>(h, mu_, t);
+    if (up > 0) {  // Y = X, taken once more with the bits that up keeps
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) fx_take_entry<N>(y, i, j, X.e[i][j].re, X.e[i][j].im, g, up);
+    }
 #pragma unroll
     for (int i = 0; i < N; ++i)
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            h.re[i][j] += (((long long)y.rh[i][j] << 29) + y.rl[i][j]) << up;
-            h.im[i][j] += (((long long)y.ih[i][j] << 29) + y.il[i][j]) << up;
+            h.re[i][j] += ((long long)y.rh[i][j] << 29) + y.rl[i][j];
+            h.im[i][j] += ((long long)y.ih[i][j] << 29) + y.il[i][j];
         }
     fx_operand_wide<N, 0>(o, h);
 #pragma unroll 1

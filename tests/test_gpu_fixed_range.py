@@ -203,3 +203,22 @@ def test_weak_sites_do_not_depend_on_the_launch(tgf):
     many.stage(1, 0.01)
     ref = one.get_links()[0]
     assert all(np.array_equal(g, ref) for g in many.get_links())
+
+
+def test_su4_exponential_keeps_small_entries(tgf):
+    """Links of large diagonal phases and off-diagonal entries of 1e-6, one stage with eps/4 = 1e-4: the force is within
+    4 U of its size (below 6) and enters with 1e-4, 2.7e-19 = 2^-61.7 off the diagonal; exp(X) - 1 is scaled to X, so that it adds no
+    2^-58 of its own.  Bar 2^-60."""
+    rng = np.random.default_rng(4)
+    ph = rng.uniform(-1, 1, (L[3], L[2], L[1], L[0], 4, 4))
+    ph -= ph.mean(-1, keepdims=True)
+    u = np.exp(1j * ph)[..., None] * I.random_links(L, 5, 1e-6, N=4)
+    b = batch(tgf, 4, [(0,) * 6])
+    b.set_links([u])
+    b.stage(1, 4e-4)
+    w = u.astype(np.clongdouble)
+    z = O.force(w, FLAT)
+    assert np.abs(z).max() < 6
+    d = b.get_links()[0].astype(np.clongdouble) - (w + np.matmul(exp_m1(1e-4 * z), w))
+    off = d[..., ~np.eye(4, dtype=bool)]
+    assert float(np.sqrt((np.abs(off) ** 2).mean() / 2)) <= 2.0 ** -60

@@ -376,18 +376,18 @@ def roofline_of(tgf, prec_name, V, stage_ms, meas_ms, workload, peaks, hbm_peak)
     launch time against the measured FMA peak of its precision; algorithmic bytes per launch over
     the same time against the measured HBM copy bandwidth.
 
-    The FP64 stage forms its products in fixed point on the integer pipe, three IMAD.WIDE per
-    multiply-add at a quarter of the FP32 FMA rate, so its denominator is the measured FP32 FMA peak / 12
-    (the FP64 FMA peak, which it exceeds, is reported beside it)."""
+    The FP64 stage forms its products in fixed point, three integer multiply-adds each, so its
+    denominator is the measured rate of those (TGF_FMA_PEAK_FIXED; the FP64 FMA peak, which it
+    exceeds, is reported beside it)."""
     stage_avg = sum(stage_ms) / 3
-    peak = peaks["fp32"] / 12 if prec_name == "fp64" else peaks["fp32"]
+    peak = peaks["fixed" if prec_name == "fp64" else "fp32"]
     achieved = STAGE_FLOP * V / (stage_avg * 1e-3) / 1e12
     alg_bytes = sum(STAGE_BYTES[prec_name]) / 3.0 * V
     gbs = alg_bytes / (stage_avg * 1e-3) / 1e9
     return {"kernel": "k_stage (fused staples+force+RK3+exp+update)", "bound": "alu",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "peak_source": "measured FP32 FMA-pipe peak (tgf_fma_peak)" + (
-                " / 12: three IMAD.WIDE per multiply-add, each at a quarter of the FMA rate" if prec_name == "fp64" else ""),
+            "peak_source": "measured %s (tgf_fma_peak)" % (
+                "integer multiply-add rate, three per fixed-point multiply-add" if prec_name == "fp64" else "FP32 FMA-pipe peak"),
             "fp64_fma_peak": peaks["fp64"],
             "traffic": stored_traffic(workload, prec_name), "traffic_unit": "DRAM bytes per stage launch (ncu, mean of stages 1-3)",
             "algorithmic_bytes_per_launch": alg_bytes, "hbm_gbs": gbs, "hbm_peak_gbs": hbm_peak,
@@ -598,7 +598,7 @@ def run_tgf(args):
 
     # ---- dominant kernel: the fused stage kernel, timed live on the same workload ------------------
     peaks = {"fp32": tgf.tgf_fma_peak(tgf.TGF_FP32), "fp64": tgf.tgf_fma_peak(tgf.TGF_FP64),
-             "fp32_packed": tgf.tgf_fma_peak(tgf.TGF_FMA_PEAK_FP32X2)}
+             "fp32_packed": tgf.tgf_fma_peak(tgf.TGF_FMA_PEAK_FP32X2), "fixed": tgf.tgf_fma_peak(tgf.TGF_FMA_PEAK_FIXED)}
     hbm = hbm_peak_gbs()
     tgf.tgf_pack(prec, b.lat, canon_dev, b.links)
     stage_ms, meas_ms = time_stages(tgf, b, args.prec, flags=flags)
@@ -727,7 +727,7 @@ def run_tgf(args):
             "gpu_launches": launches_per_flow(members) * args.steps,
             "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
             "peaks": {"fp32_fma_tflops": peaks["fp32"], "fp32_packed_fma_tflops": peaks["fp32_packed"],
-                      "fp64_fma_tflops": peaks["fp64"], "hbm_gbs": hbm},
+                      "fp64_fma_tflops": peaks["fp64"], "fixed_fma_tflops": peaks["fixed"], "hbm_gbs": hbm},
             "lambda_tgf": {str(k): {"lambda": v[0], "kept": v[1]} for k, v in lam_all.items()},
             "forms": forms,
         }

@@ -87,10 +87,17 @@ typedef enum {
 } tgf_status;
 
 typedef enum {
-    TGF_FP64 = 0,     /* links, staples, exponential, X in double                     */
+    TGF_FP64 = 0,     /* links, X, scalars, sums in double; see below                 */
     TGF_FP32 = 1,     /* links (18 reals), staples, exponential, X in float; sums FP64 */
     TGF_FP32_R12 = 2  /* as TGF_FP32 with links stored as two rows (12 reals)          */
 } tgf_precision;
+/* TGF_FP64, tgf_mc_sweeps and the SU(N) calls form matrix products in 58-bit fixed point, where links are
+ * of size 1 all over: every entry is resolved to 2^-58, about 3e-17 in a link's force against 6e-17 in
+ * double arithmetic.  Links whose surroundings are near the unit matrix (every part of the links that their
+ * staples read within 2^-4 of 0 or +-1) or whose entries or sums leave the fixed-point range (entries above
+ * 1 + 2^-10, infinities, NaN) take double arithmetic throughout: small fields keep the relative precision of
+ * double, and any input is served, at a third of the speed.  tgf_mc_sweeps keeps near-unit links in fixed
+ * point, as its heat-bath draws are coarser there in double arithmetic too. */
 
 #define TGF_MAX_CFG 256
 
@@ -384,12 +391,14 @@ tgf_status tgf_slice_correlator(const double *q, size_t q_stride, const double *
  * the roofline denominator of the flow kernels, which are bound by vector FP arithmetic.  With
  * TGF_FMA_PEAK_FP32X2 the same chains run as packed fma.rn.f32x2 pairs, with
  * TGF_FMA_PEAK_FP32_MIXED as packed and scalar FMAs interleaved: the FP32 flow kernels use
- * packed pairs, so these check that no mix of the two forms exceeds the scalar FP32 peak.  The
- * paper has no counterpart; this is a measurement aid.  `sink_dev` is a caller-owned device
+ * packed pairs, so these check that no mix of the two forms exceeds the scalar FP32 peak.  With
+ * TGF_FMA_PEAK_FIXED they run as 32 x 32 + 64 bit integer multiply-adds, counted as 2 flops per
+ * three: the rate of the FP64 kernels' fixed-point products.  The paper has no counterpart; this is a measurement aid.  `sink_dev` is a caller-owned device
  * buffer of at least blocks_per_sm * (number of SMs) * 8 bytes that the kernel may write;
  * the call synchronises `stream`. */
 #define TGF_FMA_PEAK_FP32X2 3
 #define TGF_FMA_PEAK_FP32_MIXED 4
+#define TGF_FMA_PEAK_FIXED 5
 tgf_status tgf_fma_peak(int prec, void *sink_dev, int blocks_per_sm, int iters, double *tflops,
                         void *stream);
 

@@ -23,7 +23,7 @@ TGF_NO_GRAPH = 2
 TGF_SYNC = 4
 TGF_ANY_EXTENTS = 1
 TGF_MAX_CFG = 256
-TGF_FMA_PEAK_FP32X2, TGF_FMA_PEAK_FP32_MIXED = 3, 4
+TGF_FMA_PEAK_FP32X2, TGF_FMA_PEAK_FP32_MIXED, TGF_FMA_PEAK_FIXED = 3, 4, 5
 PRECISIONS = {"fp64": TGF_FP64, "fp32": TGF_FP32, "fp32_r12": TGF_FP32_R12}
 
 

@@ -6,7 +6,8 @@
 // caller-owned sink so the chains cannot be removed.  The packed FP32 variant runs the same
 // chains on fma.rn.f32x2 pairs (two FMAs per instruction): it checks that the packed form the
 // FP32 flow kernels use does not deliver more than the scalar peak, which would make that the
-// roofline denominator instead.
+// roofline denominator instead.  The fixed-point variant runs the chains on 32 x 32 + 64 bit integer multiply-adds,
+// three of which make one multiply-add of the FP64 forms' products (fixed.cuh).
 #include <cuda_runtime.h>
 
 #include "../../include/tgf.h"
@@ -89,11 +90,36 @@ __global__ void __launch_bounds__(256) k_fma_mixed(float* sink, int iters, float
     if (s == -12345.678f) sink[blockIdx.x] = s;
 }
 
+// 8 independent chains of 32 x 32 + 64 bit multiply-adds, as the kernels' sums of products; the factor is opaque in every row,
+// so that no product is formed once and added again
+__global__ void __launch_bounds__(256) k_mad_wide(long long* sink, int iters, int b) {
+    long long x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = (long long)threadIdx.x + k;
+    int a = b ^ (int)threadIdx.x, c[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) c[k] = b + k * 0x1234567;
+#pragma unroll 1
+    for (int i = 0; i < iters; ++i) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            asm volatile("" : "+r"(a));
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] += (long long)a * c[k];
+        }
+    }
+    long long s = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s ^= x[k];
+    if (s == -1234567890123ll) sink[blockIdx.x] = s;
+}
+
 }  // namespace
 
 extern "C" tgf_status tgf_fma_peak(int prec, void* sink_dev, int blocks_per_sm, int iters, double* tflops,
                                    void* stream) {
-    if ((prec != TGF_FP64 && prec != TGF_FP32 && prec != TGF_FMA_PEAK_FP32X2 && prec != TGF_FMA_PEAK_FP32_MIXED) ||
+    if ((prec != TGF_FP64 && prec != TGF_FP32 && prec != TGF_FMA_PEAK_FP32X2 && prec != TGF_FMA_PEAK_FP32_MIXED &&
+         prec != TGF_FMA_PEAK_FIXED) ||
         !sink_dev || blocks_per_sm < 1 || iters < 1 || !tflops)
         return TGF_EINVAL;
     int dev = 0, nsm = 0;
@@ -110,6 +136,8 @@ extern "C" tgf_status tgf_fma_peak(int prec, void* sink_dev, int blocks_per_sm, 
             k_fma_x2<<<grid, 256, 0, st>>>((float*)sink_dev, iters, 0.999999f, 1e-9f);
         else if (prec == TGF_FMA_PEAK_FP32_MIXED)
             k_fma_mixed<<<grid, 256, 0, st>>>((float*)sink_dev, iters, 0.999999f, 1e-9f);
+        else if (prec == TGF_FMA_PEAK_FIXED)
+            k_mad_wide<<<grid, 256, 0, st>>>((long long*)sink_dev, iters, 0x12345677);
         else
             k_fma<float><<<grid, 256, 0, st>>>((float*)sink_dev, iters, 0.999999f, 1e-9f);
     };
@@ -123,7 +151,9 @@ extern "C" tgf_status tgf_fma_peak(int prec, void* sink_dev, int blocks_per_sm, 
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (err != cudaSuccess || ms <= 0.f) return TGF_ECUDA;
-    const double fmas_per_row = prec == TGF_FMA_PEAK_FP32X2 ? 16.0 : prec == TGF_FMA_PEAK_FP32_MIXED ? 24.0 : 8.0;
+    const double fmas_per_row = prec == TGF_FMA_PEAK_FP32X2 ? 16.0 : prec == TGF_FMA_PEAK_FP32_MIXED ? 24.0
+                                : prec == TGF_FMA_PEAK_FIXED                                            ? 8.0 / 3.0
+                                                                                                        : 8.0;
     const double flops = 2.0 * fmas_per_row * 16.0 * (double)iters * 256.0 * (double)grid;
     *tflops = flops / (ms * 1e-3) / 1e12;
     return TGF_OK;

@@ -1,11 +1,11 @@
 // fixed.cuh -- products of unitary matrices in 58-bit fixed point on the integer pipe.
 //
 // Why.  GB300 issues a warp's FP64 FMA every 64 cycles per SM quarter, but a 32 x 32 + 64 -> 64 bit
-// integer multiply-add (IMAD.WIDE) every 4 (measured: 1.90 and 29 lanes per clock and SM).
+// integer multiply-add (IMAD.WIDE) every 4 (tgf_fma_peak: 2.0 and 31.9 lanes per clock and SM).
 // Entries of SU(N) matrices are at most 1, so they need no exponent: an entry is the integer
 // v = floor(x 2^58), split as v = hi 2^29 + lo with 0 <= lo < 2^29, and one multiply-add of two
 // entries is three IMAD.WIDE (hi hi; hi lo and lo hi, summed apart; lo lo is below the last bit kept):
-// 13 cycles instead of 64.
+// 12 cycles instead of 64.
 //
 // Accuracy.  Operands of 2^-5 and more are exact, smaller ones are cut towards 0 at 2^-58.  Sums are exact: rounding
 // enters once per entry and product, when the sum of the cross terms is rounded to 2^-58 (half a unit at most) and

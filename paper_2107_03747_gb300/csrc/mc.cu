@@ -277,7 +277,8 @@ __device__ __forceinline__ void native_update(double* __restrict__ base, int Vp,
 // conversion of the result: about 130 FP64 instructions instead of 2,200, which kept the FP64 pipe 94 % busy.
 // W rotated in FP64 put 210 there, in three chains that nothing overlaps.
 // One hybrid sweep (1 heat-bath, 12 over-relaxation) of 256 x 4x4x12x12: 114.9 ms in FP64, 33.2 with W rotated in
-// FP64, 31.7 now; of 60 such fields 9.93 -> 9.06, of 8 3.76 -> 3.47.  The integer pipe is about 66 % busy; with 168 registers an SM holds
+// FP64, 31.7 in fixed point, 31.4 now; of 60 such fields 9.93 -> 9.06 -> 9.01, of 8 3.76 -> 3.47 -> 3.41.
+// The integer multiply pipe is about 63 % busy; with 168 registers an SM holds
 // 12 warps, and 4 blocks of it spill (35.8 ms).
 template <int OVERRELAX, int CAP>
 __global__ void __launch_bounds__(kMcThreads, 3) k_mc(const __grid_constant__ BatchT<CAP> B, double* __restrict__ w,

@@ -4,11 +4,11 @@
 //
 // With everything in FP64 the stage kept the FP64 pipe 94-97 % busy (107,000 cycles per warp and SM
 // quarter), and nothing else of the chip was in use.  Here that pipe carries about 115 instructions (7,200
-// cycles) and the integer pipe 13 products (4,900 IMAD.WIDE of 4 cycles) and the splitting of the operands:
-// 34,000 cycles, the multiply pipe 65 % busy.  4 steps of 4 x 8x8x24x24, measured each step: 23.8 ms before,
+// cycles) and the integer pipe 13 products (4,500 IMAD.WIDE of 4 cycles) and the splitting of the operands:
+// 34,000 cycles, the multiply pipe 53 % busy.  4 steps of 4 x 8x8x24x24, measured each step: 23.8 ms before,
 // 8.6 with the products in fixed point, 7.8 with the exponential (fx_exp_su3) as well, 7.6 with the block's
-// links taken in once and shared; one measurement of 4 x 7x7x21x21: 693 us before, 272 now; 3 steps of
-// 4x4x12x12 (latency): 696 us before, 281 now.
+// links taken in once and shared, and 7.6 with the unbiased sums and the checks that it has now; one measurement of
+// 4 x 7x7x21x21: 693 us before, 271 now; 3 steps of 4x4x12x12 (latency): 696 us before, 281 now.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -482,8 +482,8 @@ constexpr bool kSunShares = N > 2;
 
 // one RK3 stage for SU(N); block = 4 warps (one per direction) x 32 sites.  Matrix products in fixed point
 // on the integer pipe (fixed.cuh), scalars in FP64, as the SU(3) kernels of stage64.cuh; all of it in FP64 kept
-// that pipe 90-96 % busy.  Two steps and a measurement of 8 x 8x8x16x16 in SU(2): 4.08 ms before, 1.45 now; one
-// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.30 now.
+// that pipe 90-96 % busy.  Two steps and a measurement of 8 x 8x8x16x16 in SU(2): 4.08 ms before, 1.46 now; one
+// step and a measurement of 4 x 6x6x24x24 in SU(4): 12.9 ms before, 4.16 now.
 template <int N, int STAGE, int CAP>
 __global__ void __launch_bounds__(128, N == 4 ? 2 : 3)
 k_sun_stage(const __grid_constant__ BatchT<CAP> B, const double* __restrict__ w_in, double* __restrict__ w_out,
